@@ -58,9 +58,8 @@ size_t grid_vec_bytes(const vie_problem* P, int c, int nrhs, size_t elem) {
 }
 
 // Grid sizes: any n in [4, 512].  2n and 3n that factor into the codelet
-// radices (2, 3, 5, 7, 11) take direct transforms, others Bluestein's; at
-// n = 512 the set-up holds about 100 GB on the device, and an allocation that
-// fails returns VIE_ENOMEM.
+// radices (2, 3, 5, 7, 11) take direct transforms, others Bluestein's; an
+// allocation that fails returns VIE_ENOMEM.
 static bool valid_size(int n) { return n >= 4 && n <= 512; }
 
 int conv_half(int n) {
@@ -85,7 +84,7 @@ static void free_problem(vie_problem* P) {
   if (!P) return;
   cudaStream_t st = P->stream;
   void* ptrs[] = {P->tw64, P->tw32, P->He64, P->He32, P->Hm64, P->Hm32, P->twdf, P->Hedf, P->Hmdf,
-                  P->sym_oct, P->ws.buf, P->ks.buf, P->dflag};
+                  P->base_oct, P->ws.buf, P->ks.buf, P->dflag};
   for (void* q : ptrs) dfree(q, st);
   free_set(P->kapply, st);
   free_set(P->keval, st);
@@ -270,7 +269,7 @@ size_t vie_problem_bytes(int kind, int n, int nrhs, int restart, int has_mu) {
   held += 16 * O3 * nsym;                    // raw symbol octants
   held += 24 * O3 * 18;                      // apply + eval kernel sets, FP64 + FP32
   held += 96 * N * (has_mu ? 2 : 1) + 16 * O3 * (kind == VIE_MAXWELL ? 9 : 6);  // double-word copies (mixed solve)
-  // set-up peak: oversampled (3n)^3 and convolution-grid (2nk)^3 FP64 transform buffers
+  // allowance for set-up scratch (the octant line operators hold less)
   const size_t setup = held + 16 * (27 * N + 8 * nk * nk * nk);
   // steady state: FP64 apply workspace, mixed-precision Krylov group
   size_t steady = held + apply_workspace_bytes(n, (int)nk, c, nrhs, VIE_FP64);

@@ -1,5 +1,5 @@
 // Set-up kernels of a problem, on the device, to FP64 accuracy (FP64 arithmetic,
-// except the kernel-transform cube FFTs, which run in double-word arithmetic on
+// except the kernel-transform line FFTs, which run in double-word arithmetic on
 // the FP32 pipes unless VIE_SETUP_FP64=1):
 //  * H_eps = (eps + I)^-1 (eps - I) per node (Eq. (rhodef), Lemma 1), stored as
 //    the 6 entries of the symmetric tensor in FP64 and FP32;
@@ -7,7 +7,7 @@
 //    tabulated once per distinct integer |m|^2 of the oversampled frequency grid;
 //  * the discrete kernels of every Fourier symbol (1, i k_a, -k_a k_b) with the
 //    grid Nyquist cutoff (Sec. 5, step c), brought to the (2n)^3 convolution
-//    grid and stored as octants (the kernels are even or odd in each axis).
+//    grid, on octants throughout (the kernels are even or odd in each axis).
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -212,163 +212,228 @@ __global__ void k_ghat_table(double2* tab, int jmax, double dk, double w, double
   tab[j] = dev_ghat(dk * sqrt((double)j), w, L);
 }
 
-// F(m) = S~(k_m) G^(|k_m|) on the (sn)^3 grid in FFT order.  Even sn: m in
-// [-sn/2, sn/2), and on an axis with m_a = -sn/2 (Nyquist) an odd factor k_a is
-// replaced by 0 (the mean of its values at -pi/h and +pi/h), an even factor k_a^2
-// is kept.  Odd sn (odd n): m in [-(sn-1)/2, (sn-1)/2], no Nyquist entry.  Either
-// way |m_a| <= sn/2 (integer division), so m.m <= 3 (sn/2)^2, the table's length.
-__global__ void k_build_F(double2* __restrict__ F, const double2* __restrict__ tab, int sn, int sym, double dk) {
-  const long long tot = (long long)sn * sn * sn;
-  const int hp = (sn + 1) / 2;                // first index of a negative m
-  const int nyq = (sn % 2 == 0) ? sn / 2 : -1;  // index of m = -sn/2, if any
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < tot;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(idx % sn);
-    const int iy = (int)((idx / sn) % sn);
-    const int iz = (int)(idx / ((long long)sn * sn));
-    const int mx = ix < hp ? ix : ix - sn, my = iy < hp ? iy : iy - sn, mz = iz < hp ? iz : iz - sn;
-    const long long j = (long long)mx * mx + (long long)my * my + (long long)mz * mz;
-    const double2 G = tab[j];
-    const double kx = dk * mx, ky = dk * my, kz = dk * mz;
-    const double ox = (ix == nyq) ? 0.0 : kx, oy = (iy == nyq) ? 0.0 : ky, oz = (iz == nyq) ? 0.0 : kz;
-    double2 v;
-    switch (sym) {
-      case SYM_1: v = G; break;
-      case SYM_DX: v = make_double2(-ox * G.y, ox * G.x); break;
-      case SYM_DY: v = make_double2(-oy * G.y, oy * G.x); break;
-      case SYM_DZ: v = make_double2(-oz * G.y, oz * G.x); break;
-      case SYM_XX: v = (-kx * kx) * G; break;
-      case SYM_YY: v = (-ky * ky) * G; break;
-      case SYM_ZZ: v = (-kz * kz) * G; break;
-      case SYM_XY: v = (-ox * oy) * G; break;
-      case SYM_XZ: v = (-ox * oz) * G; break;
-      default: v = (-oy * oz) * G; break;
-    }
-    F[idx] = v;
+// The discrete kernels.  On the (sn)^3 frequency grid F(m) = S~(k_m) G^(|k_m|)
+// depends on m only through |m_x|, |m_y|, |m_z| and one sign per axis (a factor
+// k_a is odd in m_a, everything else is even), and "inverse DFT over sn, keep the
+// offsets |d| < n, place them at d mod M, DFT over M" acts on each axis by
+// itself, keeping that parity.  So a symbol's octant (nk + 1)^3 comes from the
+// octant m >= 0 of F by one line operator per axis, x, y, z in turn, each in a
+// single pass that reads sn/2 + 1 entries of a line and writes nk + 1: 4.75 n^2
+// lines of sn and M points, against 27 n^2 and 12 n^2 for the whole cubes, and
+// 10 n^3 against 210 n^3 values moved.  All symbols follow from four of them by
+// exchanging axes (G^ is radial): 1, -k_z^2, -k_x k_y and i k_z, z being the
+// axis that is not like the other two.
+// Measured, 192^3 reduced Maxwell problem: 302 ms for seven symbols on whole cubes
+// (279 ms of cube transforms, 21 ms to fill them), 29.5 ms for three bases here.
+enum Base { BASE_1 = 0, BASE_ZZ, BASE_XY, BASE_DZ, BASE_COUNT };
+
+static int base_of(int sym) {
+  switch (sym) {
+    case SYM_1: return BASE_1;
+    case SYM_XX: case SYM_YY: case SYM_ZZ: return BASE_ZZ;
+    case SYM_XY: case SYM_XZ: case SYM_YZ: return BASE_XY;
+    default: return BASE_DZ;
+  }
+}
+// Axis of the symbol that takes the place of its base's z (2 z, 1 y, 0 x).
+static int axis_of(int sym) {
+  switch (sym) {
+    case SYM_XX: case SYM_YZ: case SYM_DX: return 0;
+    case SYM_YY: case SYM_XZ: case SYM_DY: return 1;
+    default: return 2;
   }
 }
 
-// Generic in-place FFT of a cubic M^3 FP64 array along one axis (0 x, 1 y, 2 z).
-template <int S, typename T>
-__global__ void k_fft_cube(double2* __restrict__ data, int M, int axis, FftPlan pl,
-                           const typename CT<T>::V* __restrict__ twg, int nl) {
+struct AxisPass {
+  int axis;        // 0 x, 1 y, 2 z
+  int base;        // Base
+  int n, nk, sn;
+  int odd;         // the base is odd in this axis
+  int nl;          // lines per tile
+  int LS;          // pitch of a tile line
+  double dk;       // frequency spacing 2 pi / (3 D)
+  double scale;    // factor of the stored values (1, or 1/(sn)^3 in the last pass)
+  FftPlan ps, pm;  // line plans of lengths sn and M = 2 nk
+};
+
+// F of base `b` at m >= 0 (all axes).  Even sn: m_a = sn/2 is the Nyquist entry,
+// where an odd factor k_a is replaced by 0 (the mean of its values at -pi/h and
+// +pi/h) and an even factor k_a^2 is kept.  Odd sn has no Nyquist entry.
+__device__ __forceinline__ double2 base_sample(const double2* __restrict__ tab, int b, int mx, int my, int mz, int sn,
+                                               double dk) {
+  const double2 G = tab[mx * mx + my * my + mz * mz];
+  auto kodd = [&](int m) { return 2 * m == sn ? 0.0 : dk * m; };
+  if (b == BASE_1) return G;
+  if (b == BASE_ZZ) return (-(dk * mz) * (dk * mz)) * G;
+  if (b == BASE_XY) return (-kodd(mx) * kodd(my)) * G;
+  const double oz = kodd(mz);
+  return make_double2(-oz * G.y, oz * G.x);
+}
+
+// One line operator over `nl` lines per CTA (blockDim.y = nl, blockDim.x threads
+// a line).  Layouts: x pass  tab -> out [mz][my][kx], y pass [mz][my][kx] ->
+// [mz][ky][kx], z pass [mz][ky][kx] -> [kz][ky][kx]; 0 <= m <= sn/2, 0 <= k <= nk.
+// The lines of a y or z tile are neighbours in kx, so a tile reads and writes
+// runs of nl 16-byte values.
+template <typename T>
+__global__ void k_axis(const double2* __restrict__ in, double2* __restrict__ out, AxisPass q,
+                       const typename CT<T>::V* __restrict__ tws, const typename CT<T>::V* __restrict__ twm) {
   typedef typename CT<T>::V V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int Q = pl.Q, LS = Q + 1;
-  V* tw = (V*)smraw;
-  V* b0 = tw + Q;
+  const int nl = q.nl, LS = q.LS, sn = q.sn, n = q.n, M = q.pm.M, Q = q.ps.Q, O = q.nk + 1, S = sn / 2 + 1;
+  V* ts = (V*)smraw;
+  V* tm = ts + Q;
+  V* b0 = tm + M;
   V* b1 = b0 + nl * LS;
   const int tid = flat_tid(), nt = flat_nthreads();
-  for (int j = tid; j < Q; j += nt) tw[j] = twg[j];
-  const long long MM = (long long)M * M;
-  // address of element j of tile line l
-  auto addr = [&](int l, int j) -> long long {
-    if (axis == 0) return ((long long)blockIdx.x * nl + l) * M + j;
-    if (axis == 1) return (long long)blockIdx.y * MM + (long long)j * M + (long long)blockIdx.x * nl + l;
-    return (long long)j * MM + (long long)blockIdx.y * M + (long long)blockIdx.x * nl + l;
-  };
-  for (int idx = tid; idx < nl * M; idx += nt) {
-    int l, j;
-    if (axis == 0) { l = idx / M; j = idx - l * M; } else { j = idx / nl; l = idx - j * nl; }
-    b0[l * LS + j] = to_v<T>(data[addr(l, j)]);
+  for (int j = tid; j < Q; j += nt) ts[j] = tws[j];
+  for (int j = tid; j < M; j += nt) tm[j] = twm[j];
+  // lines of this tile: x pass rows r0 + l < S^2; y, z passes kx = r0 + l < O of slab blockIdx.y
+  const int r0 = blockIdx.x * nl, slab = blockIdx.y;
+  const long long lines = q.axis == 0 ? (long long)S * S : O;
+  // stride between entries of a line, and the first entry of line r, on the input and output side
+  const long long istep = q.axis == 1 ? O : (long long)O * O;
+  const long long ibase = q.axis == 1 ? (long long)slab * S * O : (long long)slab * O;
+  const long long ostep = q.axis == 0 ? 1 : istep;
+  const long long obase = q.axis == 1 ? (long long)slab * O * O : (long long)slab * O;
+  for (int idx = tid; idx < nl * S; idx += nt) {
+    int l, m;
+    if (q.axis == 0) { l = idx / S; m = idx - l * S; } else { m = idx / nl; l = idx - m * nl; }
+    const long long r = r0 + l;
+    double2 v = make_double2(0.0, 0.0);
+    if (r < lines) {
+      if (q.axis == 0) {
+        const int mz = (int)(r / S), my = (int)(r - (long long)mz * S);
+        v = base_sample(in, q.base, m, my, mz, sn, q.dk);
+      } else {
+        v = in[ibase + m * istep + r];
+      }
+    }
+    const V a = to_v<T>(v);
+    b0[l * LS + m] = a;
+    if (m > 0 && 2 * m != sn) b0[l * LS + sn - m] = q.odd ? vneg(a) : a;
   }
   __syncthreads();
-  V* r = line_fft<S, T>(b0, b1, pl, tw, twg + Q, nl, LS);
+  V* r = line_fft<+1, T>(b0, b1, q.ps, ts, tws + Q, nl, LS);
+  V* e = (r == b0) ? b1 : b0;
+  // offsets d in [-(n-1), n-1] at index d mod M, zeros between
   for (int idx = tid; idx < nl * M; idx += nt) {
-    int l, j;
-    if (axis == 0) { l = idx / M; j = idx - l * M; } else { j = idx / nl; l = idx - j * nl; }
-    data[addr(l, j)] = from_v<T>(r[l * LS + j]);
+    const int l = idx / M, j = idx - l * M;
+    e[l * LS + j] = j < n ? r[l * LS + j] : (j > M - n ? r[l * LS + j - M + sn] : CT<T>::make(0, 0));
+  }
+  __syncthreads();
+  V* w = line_fft<-1, T>(e, r, q.pm, tm, twm + M, nl, LS);
+  for (int idx = tid; idx < nl * O; idx += nt) {
+    int l, k;
+    if (q.axis == 0) { l = idx / O; k = idx - l * O; } else { k = idx / nl; l = idx - k * nl; }
+    const long long row = r0 + l;
+    if (row >= lines) continue;
+    const double2 v = from_v<T>(w[l * LS + k]);
+    out[q.axis == 0 ? row * O + k : obase + k * ostep + row] = q.scale * v;
   }
 }
 
-// Lines per tile: a power of two dividing M, with the tile within 200 KB.
-static int pick_nl(const FftPlan& pl, size_t vs) {
-  int nl = 8;
-  while (nl > 1 && (pl.M % nl != 0 || vs * (pl.Q + 2 * (size_t)nl * (pl.Q + 1)) > 200 * 1024)) nl >>= 1;
-  return nl;
-}
-
-// In-place 3D DFT of an FP64 cube, lines along each axis in turn; arithmetic in
-// T (FP64, or double-word on the FP32 pipes), one block row per tile line.
-template <int S, typename T>
-static vie_status fft_cube(double2* data, int M, const FftPlan& pl, const typename CT<T>::V* tw, cudaStream_t st) {
-  const size_t vs = sizeof(typename CT<T>::V);
-  const int nl = pick_nl(pl, vs);
-  const size_t smem = vs * (pl.Q + 2 * nl * (pl.Q + 1));
+// Octant of a base symbol: the three line operators.  A1 holds [S][S][O], A2 [S][O][O].
+template <typename T>
+static vie_status base_octant(vie_problem* P, int base, const double2* tab, double2* A1, double2* A2, double2* oct,
+                              const FftPlan& ps, const typename CT<T>::V* tws, const typename CT<T>::V* twm,
+                              cudaStream_t st) {
+  typedef typename CT<T>::V V;
+  AxisPass q;
+  q.base = base;
+  q.n = P->n;
+  q.nk = P->nk;
+  q.sn = 3 * P->n;
+  q.dk = 2.0 * M_PI / (3.0 * P->D);
+  q.ps = ps;
+  q.pm = P->planM;
+  q.LS = std::max(ps.Q, P->planM.M) + 1;
+  const int S = q.sn / 2 + 1, O = q.nk + 1;
+  // lines per tile: up to eight (128-byte runs in the y and z passes), with the
+  // tile within 110 KB, so that two CTAs share an SM, where that leaves two lines
+  auto smem_of = [&](int nl) { return sizeof(V) * (ps.Q + P->planM.M + 2 * (size_t)nl * q.LS); };
+  q.nl = 8;
+  while (q.nl > 2 && smem_of(q.nl) > 110 * 1024) q.nl >>= 1;
+  while (q.nl > 1 && smem_of(q.nl) > (size_t)smem_optin_bytes()) q.nl >>= 1;
+  const size_t smem = smem_of(q.nl);
   if (smem > (size_t)smem_optin_bytes()) {
     set_error("set-up transform line too long for shared memory");
     return VIE_EINVAL;
   }
-  VIE_CK(allow_smem(k_fft_cube<S, T>));
-  // threads per line: M/16 up to 32 for direct plans; a long Bluestein line
-  // (one to four per tile) one per 16 elements of Q, up to 128, and at most
-  // 256 threads per block
-  int tx = std::max(1, std::min(32, M / 16));
-  if (pl.Q != pl.M) {
-    tx = 32;
-    while (tx * 16 < pl.Q && tx < 128 && 2 * tx * nl <= 256) tx <<= 1;
-  }
-  const dim3 blk(tx, nl);
+  VIE_CK(allow_smem(k_axis<T>));
+  // threads a line: a power of two near Q / 8, at most 256 a block
+  int tx = 8;
+  while (tx * 8 < ps.Q && 2 * tx * q.nl <= 256) tx <<= 1;
+  const dim3 blk(tx, q.nl);
   for (int axis = 0; axis < 3; ++axis) {
-    dim3 grid = axis == 0 ? dim3((unsigned)((long long)M * M / nl), 1) : dim3(M / nl, M);
-    k_fft_cube<S, T><<<grid, blk, smem, st>>>(data, M, axis, pl, tw, nl);
+    q.axis = axis;
+    q.odd = (base == BASE_XY && axis != 2) || (base == BASE_DZ && axis == 2);
+    q.scale = axis == 2 ? 1.0 / ((double)q.sn * q.sn * q.sn) : 1.0;
+    const double2* src = axis == 0 ? tab : (axis == 1 ? A1 : A2);
+    double2* dst = axis == 0 ? A1 : (axis == 1 ? A2 : oct);
+    const dim3 grid = axis == 0 ? dim3((unsigned)(((long long)S * S + q.nl - 1) / q.nl))
+                                : dim3((O + q.nl - 1) / q.nl, axis == 1 ? S : O);
+    k_axis<T><<<grid, blk, smem, st>>>(src, dst, q, tws, twm);
     VIE_CK(cudaGetLastError());
   }
   return VIE_OK;
 }
 
-// e[M^3] (M = 2 nk >= 2n) from the inverse-transformed F[(sn)^3]: offsets d in
-// [-(n-1), n-1] at index d mod M, indices n..M-n left zero; scale folds the
-// 1/(sn)^3 of the inverse DFT.
-__global__ void k_embed(const double2* __restrict__ F, double2* __restrict__ e, int n, int nk, int sn, double scale) {
-  const int M = 2 * nk;
-  const long long tot = (long long)M * M * M;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < tot;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int ex = (int)(idx % M), ey = (int)((idx / M) % M), ez = (int)(idx / ((long long)M * M));
-    if ((ex >= n && ex <= M - n) || (ey >= n && ey <= M - n) || (ez >= n && ez <= M - n)) {
-      e[idx] = make_double2(0.0, 0.0);
-      continue;
-    }
-    const int sx = ex < n ? ex : ex - M + sn;
-    const int sy = ey < n ? ey : ey - M + sn;
-    const int sz = ez < n ? ez : ez - M + sn;
-    e[idx] = scale * F[((long long)sz * sn + sy) * sn + sx];
-  }
-}
-
-__global__ void k_octant(const double2* __restrict__ E, double2* __restrict__ oct, int nk) {
-  const int M = 2 * nk, O = nk + 1;
-  const long long tot = (long long)O * O * O;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < tot;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int ox = (int)(idx % O), oy = (int)((idx / O) % O), oz = (int)(idx / ((long long)O * O));
-    oct[idx] = E[((long long)oz * M + oy) * M + ox];
-  }
-}
-
-// Combine raw symbol octants into the kernel arrays of one pass.
-//   coef layout per output array a: up to 2 terms (sym index, complex factor).
+// Combine base octants into the kernel arrays of one pass.
+//   coef layout per output array a: up to 2 terms (base octant, the axis that
+//   takes its z, complex factor); base < 0: no term.
 struct CombineDesc {
   int narr;
-  int sym[9][2];
+  int base[9][2];
+  int axis[9][2];
   double2 fac[9][2];
+  void set(int a, int t, int sym, double2 f) {
+    base[a][t] = base_of(sym);
+    axis[a][t] = axis_of(sym);
+    fac[a][t] = f;
+  }
 };
 
-__global__ void k_combine(const double2* __restrict__ sym_oct, double2* __restrict__ out64, float2* __restrict__ out32,
-                          long long O3, CombineDesc cd, double diag_add_scale, int diag_mask) {
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < O3;
-       idx += (long long)gridDim.x * blockDim.x) {
-    for (int a = 0; a < cd.narr; ++a) {
-      double2 v = make_double2(0.0, 0.0);
-      for (int t = 0; t < 2; ++t) {
-        const int s = cd.sym[a][t];
-        if (s < 0) continue;
-        v = v + cmul(cd.fac[a][t], sym_oct[(long long)s * O3 + idx]);
+// The bases are symmetric under exchange of their x and y, so a symbol whose
+// odd-one-out axis is z or y reads base[oz][oy][ox] or base[oy][oz][ox], both
+// contiguous in ox, and one whose axis is x reads base[ox][oz][oy], which a
+// 32 x 32 tile in shared memory turns round.  grid = (ox tiles, oy tiles, oz).
+__global__ void __launch_bounds__(256) k_combine(const double2* __restrict__ bases, double2* __restrict__ out64,
+                                                 float2* __restrict__ out32, int O, CombineDesc cd,
+                                                 double diag_add_scale, int diag_mask) {
+  __shared__ double2 tile[32][33];
+  const long long O3 = (long long)O * O * O;
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, oz = blockIdx.z;
+  for (int a = 0; a < cd.narr; ++a) {
+    double2 v[4];
+    for (int i = 0; i < 4; ++i) v[i] = make_double2(0.0, 0.0);
+    for (int t = 0; t < 2; ++t) {
+      const int bs = cd.base[a][t], ax = cd.axis[a][t];
+      if (bs < 0) continue;  // uniform over the grid
+      const double2* src = bases + bs * O3;
+      if (ax == 0) {
+        __syncthreads();
+        for (int i = 0; i < 4; ++i) {
+          const int ox = x0 + threadIdx.y + 8 * i, oy = y0 + threadIdx.x;
+          if (ox < O && oy < O) tile[threadIdx.y + 8 * i][threadIdx.x] = src[((long long)ox * O + oz) * O + oy];
+        }
+        __syncthreads();
       }
-      if (diag_mask & (1 << a)) v.x += diag_add_scale;
-      out64[a * O3 + idx] = v;
-      out32[a * O3 + idx] = make_float2((float)v.x, (float)v.y);
+      for (int i = 0; i < 4; ++i) {
+        const int ox = x0 + threadIdx.x, oy = y0 + threadIdx.y + 8 * i;
+        if (ox >= O || oy >= O) continue;
+        const double2 s = ax == 0 ? tile[threadIdx.x][threadIdx.y + 8 * i]
+                                  : src[ax == 1 ? ((long long)oy * O + oz) * O + ox : ((long long)oz * O + oy) * O + ox];
+        v[i] = v[i] + cmul(cd.fac[a][t], s);
+      }
+    }
+    for (int i = 0; i < 4; ++i) {
+      const int ox = x0 + threadIdx.x, oy = y0 + threadIdx.y + 8 * i;
+      if (ox >= O || oy >= O) continue;
+      if (diag_mask & (1 << a)) v[i].x += diag_add_scale;
+      const long long idx = a * O3 + ((long long)oz * O + oy) * O + ox;
+      out64[idx] = v[i];
+      out32[idx] = make_float2((float)v[i].x, (float)v[i].y);
     }
   }
 }
@@ -380,43 +445,45 @@ static vie_status combine(vie_problem* P, KernelSet& K, int mode, const CombineD
   K.narr = cd.narr;
   VIE_CK(dalloc((void**)&K.oct64, sizeof(double2) * cd.narr * O3, st));
   VIE_CK(dalloc((void**)&K.oct32, sizeof(float2) * cd.narr * O3, st));
-  const int blocks = (int)std::min<long long>((O3 + 255) / 256, 152LL * 16);
-  k_combine<<<blocks, 256, 0, st>>>(P->sym_oct, K.oct64, K.oct32, O3, cd, diag_add, diag_mask);
+  const unsigned tiles = (unsigned)((O + 31) / 32);
+  k_combine<<<dim3(tiles, tiles, (unsigned)O), dim3(32, 8), 0, st>>>(P->base_oct, K.oct64, K.oct32, (int)O, cd,
+                                                                     diag_add, diag_mask);
   VIE_CK(cudaGetLastError());
   return VIE_OK;
 }
 
-// Compute the raw octant kernels of the symbols in `mask` (bit = Sym) that are
-// not computed yet.
 static vie_status to_df(const double2* src, cdf** dst, long long count, cudaStream_t st);
 
-static vie_status compute_symbols(vie_problem* P, unsigned mask, cudaStream_t st) {
-  mask &= ~P->sym_mask;
+// Compute the base octants that the symbols in `syms` (bit = Sym) need and that
+// are not there yet.
+static vie_status compute_symbols(vie_problem* P, unsigned syms, cudaStream_t st) {
+  unsigned mask = 0;
+  for (int s = 0; s < SYM_COUNT; ++s)
+    if (syms & (1u << s)) mask |= 1u << base_of(s);
+  mask &= ~P->base_mask;
   if (!mask) return VIE_OK;
-  const int n = P->n, sn = 3 * n, M = 2 * P->nk;
+  const int n = P->n, sn = 3 * n;
   const double dk = 2.0 * M_PI / (3.0 * P->D);
   const int jmax = 3 * (sn / 2) * (sn / 2);
   const double w = P->kind == VIE_LAPLACE ? 0.0 : P->omega;
-  double2* tab = nullptr;
-  double2 *F = nullptr, *E = nullptr, *tw_sn = nullptr;
-  float2* tw_sn32 = nullptr;
   FftPlan plsn;
   if (!make_line_plan(sn, &plsn)) {
     set_error("bad oversampled grid size");
     return VIE_EINVAL;
   }
-  const long long O = P->nk + 1;
-  const long long S3 = (long long)sn * sn * sn, M3 = (long long)M * M * M, O3 = O * O * O;
-  if (!P->sym_oct) VIE_CK(dalloc((void**)&P->sym_oct, sizeof(double2) * SYM_COUNT * O3, st));
+  double2 *tab = nullptr, *A1 = nullptr, *A2 = nullptr, *tw_sn = nullptr;
+  float2* tw_sn32 = nullptr;
+  const long long O = P->nk + 1, S = sn / 2 + 1, O3 = O * O * O;
+  if (!P->base_oct) VIE_CK(dalloc((void**)&P->base_oct, sizeof(double2) * BASE_COUNT * O3, st));
   VIE_CK(dalloc((void**)&tab, sizeof(double2) * (jmax + 1), st));
   k_ghat_table<<<(jmax + 256) / 256, 256, 0, st>>>(tab, jmax, dk, w, P->L);
   VIE_CK(cudaGetLastError());
-  VIE_CK(dalloc((void**)&F, sizeof(double2) * S3, st));
-  VIE_CK(dalloc((void**)&E, sizeof(double2) * M3, st));
+  VIE_CK(dalloc((void**)&A1, sizeof(double2) * S * S * O, st));
+  VIE_CK(dalloc((void**)&A2, sizeof(double2) * S * O * O, st));
   vie_status s = make_line_table(plsn, &tw_sn, &tw_sn32, st);
   if (s != VIE_OK) return s;
-  // the kernel-transform FFTs run in double-word arithmetic (FP64 accuracy on
-  // the FP32 pipes); VIE_SETUP_FP64=1 keeps them in native FP64
+  // the transforms run in double-word arithmetic (FP64 accuracy on the FP32
+  // pipes); VIE_SETUP_FP64=1 keeps them in native FP64
   const char* e64 = getenv("VIE_SETUP_FP64");
   const bool dw = !(e64 && e64[0] == '1');
   cdf *tw_sndf = nullptr, *tw_2ndf = nullptr;
@@ -425,28 +492,21 @@ static vie_status compute_symbols(vie_problem* P, unsigned mask, cudaStream_t st
     if (s == VIE_OK) s = to_df(P->tw64, &tw_2ndf, line_table_len(P->planM), st);
     if (s != VIE_OK) return s;
   }
-  const int gb = 152 * 16;
-  for (int sym = 0; sym < SYM_COUNT; ++sym) {
-    if (!(mask & (1u << sym))) continue;
-    k_build_F<<<gb, 256, 0, st>>>(F, tab, sn, sym, dk);
-    VIE_CK(cudaGetLastError());
-    s = dw ? fft_cube<+1, df>(F, sn, plsn, tw_sndf, st) : fft_cube<+1, double>(F, sn, plsn, tw_sn, st);
+  for (int b = 0; b < BASE_COUNT; ++b) {
+    if (!(mask & (1u << b))) continue;
+    double2* oct = P->base_oct + b * O3;
+    s = dw ? base_octant<df>(P, b, tab, A1, A2, oct, plsn, tw_sndf, tw_2ndf, st)
+           : base_octant<double>(P, b, tab, A1, A2, oct, plsn, tw_sn, P->tw64, st);
     if (s != VIE_OK) return s;
-    k_embed<<<gb, 256, 0, st>>>(F, E, n, P->nk, sn, 1.0 / (double)S3);
-    VIE_CK(cudaGetLastError());
-    s = dw ? fft_cube<-1, df>(E, M, P->planM, tw_2ndf, st) : fft_cube<-1, double>(E, M, P->planM, P->tw64, st);
-    if (s != VIE_OK) return s;
-    k_octant<<<gb, 256, 0, st>>>(E, P->sym_oct + (long long)sym * O3, P->nk);
-    VIE_CK(cudaGetLastError());
   }
-  dfree(F, st);
-  dfree(E, st);
+  dfree(A1, st);
+  dfree(A2, st);
   dfree(tab, st);
   dfree(tw_sn, st);
   dfree(tw_sn32, st);
   dfree(tw_sndf, st);
   dfree(tw_2ndf, st);
-  P->sym_mask |= mask;
+  P->base_mask |= mask;
   return VIE_OK;
 }
 
@@ -538,8 +598,8 @@ static vie_status combine_sets(vie_problem* P, int which, cudaStream_t st) {
   CombineDesc ca{}, ce{};
   for (int a = 0; a < 9; ++a)
     for (int t = 0; t < 2; ++t) {
-      ca.sym[a][t] = -1;
-      ce.sym[a][t] = -1;
+      ca.base[a][t] = -1;
+      ce.base[a][t] = -1;
       ca.fac[a][t] = make_double2(0, 0);
       ce.fac[a][t] = make_double2(0, 0);
     }
@@ -550,8 +610,7 @@ static vie_status combine_sets(vie_problem* P, int which, cudaStream_t st) {
     const double sg = P->kind == VIE_LAPLACE ? -2.0 : 2.0;
     ca.narr = 6;
     for (int a = 0; a < 6; ++a) {
-      ca.sym[a][0] = Q[a];
-      ca.fac[a][0] = make_double2(sg * nrm, 0);
+      ca.set(a, 0, Q[a], make_double2(sg * nrm, 0));
     }
     if (which == 0) {
       s = combine(P, P->kapply, KM_SYM3, ca, sg * 0.5 * nrm, 0x7, st);
@@ -560,8 +619,7 @@ static vie_status combine_sets(vie_problem* P, int which, cudaStream_t st) {
     // phi_sc = div V J
     ce.narr = 3;
     for (int a = 0; a < 3; ++a) {
-      ce.sym[a][0] = Dd[a];
-      ce.fac[a][0] = make_double2(nrm, 0);
+      ce.set(a, 0, Dd[a], make_double2(nrm, 0));
     }
     if (which == 1) {
       s = combine(P, P->keval, KM_DIV, ce, 0.0, 0, st);
@@ -572,16 +630,13 @@ static vie_status combine_sets(vie_problem* P, int which, cudaStream_t st) {
     // Q' = -2 (K + I/2 + w^2 V), P'_a = -2 i w K_{i k_a}.
     ca.narr = P->has_mu ? 9 : 6;
     for (int a = 0; a < 6; ++a) {
-      ca.sym[a][0] = Q[a];
-      ca.fac[a][0] = make_double2(-2.0 * nrm, 0);
+      ca.set(a, 0, Q[a], make_double2(-2.0 * nrm, 0));
       if (a < 3) {
-        ca.sym[a][1] = SYM_1;
-        ca.fac[a][1] = make_double2(-2.0 * w2 * nrm, 0);
+        ca.set(a, 1, SYM_1, make_double2(-2.0 * w2 * nrm, 0));
       }
     }
     for (int a = 0; a < 3; ++a) {
-      ca.sym[6 + a][0] = Dd[a];
-      ca.fac[6 + a][0] = make_double2(0, -2.0 * w * nrm);
+      ca.set(6 + a, 0, Dd[a], make_double2(0, -2.0 * w * nrm));
     }
     if (which == 0) {
       s = combine(P, P->kapply, P->has_mu ? KM_MAXWELL6 : KM_SYM3, ca, -nrm, 0x7, st);
@@ -590,16 +645,13 @@ static vie_status combine_sets(vie_problem* P, int which, cudaStream_t st) {
     // E_sc = Q'' J + P'' x M, H_sc = Q'' M - P'' x J; Q'' = K + w^2 V, P''_a = i w K_{i k_a}
     ce.narr = 9;
     for (int a = 0; a < 6; ++a) {
-      ce.sym[a][0] = Q[a];
-      ce.fac[a][0] = make_double2(nrm, 0);
+      ce.set(a, 0, Q[a], make_double2(nrm, 0));
       if (a < 3) {
-        ce.sym[a][1] = SYM_1;
-        ce.fac[a][1] = make_double2(w2 * nrm, 0);
+        ce.set(a, 1, SYM_1, make_double2(w2 * nrm, 0));
       }
     }
     for (int a = 0; a < 3; ++a) {
-      ce.sym[6 + a][0] = Dd[a];
-      ce.fac[6 + a][0] = make_double2(0, w * nrm);
+      ce.set(6 + a, 0, Dd[a], make_double2(0, w * nrm));
     }
     if (which == 1) {
       s = combine(P, P->keval, P->has_mu ? KM_MAXWELL6 : KM_EMRED, ce, 0.0, 0, st);

@@ -86,8 +86,8 @@ struct vie_problem {
   vie::cdf* twdf = nullptr;  // double-word copies of tw64, He64, Hm64 (first VIE_DF64 apply)
   vie::cdf* Hedf = nullptr;
   vie::cdf* Hmdf = nullptr;
-  double2* sym_oct = nullptr;  // [SYM_COUNT][(n+1)^3] raw symbol kernels DFT_{2n}, FP64
-  unsigned sym_mask = 0;       // symbols computed so far
+  double2* base_oct = nullptr;  // [4][(nk+1)^3] raw kernels of the base symbols (precompute.cu), FP64
+  unsigned base_mask = 0;       // base symbols computed so far
   vie::KernelSet kapply;     // operator kernels (with I/2, 2H sign and 1/(2n)^3 folded in)
   vie::KernelSet keval;      // scattered-field kernels
   vie::Workspace ws;         // padded intermediates
