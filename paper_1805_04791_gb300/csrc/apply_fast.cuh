@@ -1409,9 +1409,9 @@ __global__ void __launch_bounds__(256) f_p5(const typename CT<T>::V* __restrict_
         typename IOT<T>::E* yo = y + ((long long)b * CO + 3 * blk) * N + pt;
         const V a0 = uo[3 * blk][n1], a1 = uo[3 * blk + 1][n1], a2 = uo[3 * blk + 2][n1];
         if (with_identity == 1) {
-          yo[0] = from_v<T>(to_v<T>(xi[0]) + cmul(hxx, a0) + cmul(hxy, a1) + cmul(hxz, a2));
-          yo[N] = from_v<T>(to_v<T>(xi[N]) + cmul(hxy, a0) + cmul(hyy, a1) + cmul(hyz, a2));
-          yo[2 * N] = from_v<T>(to_v<T>(xi[2 * N]) + cmul(hxz, a0) + cmul(hyz, a1) + cmul(hzz, a2));
+          yo[0] = add_id<T>(xi[0], cmul(hxx, a0), cmul(hxy, a1), cmul(hxz, a2));
+          yo[N] = add_id<T>(xi[N], cmul(hxy, a0), cmul(hyy, a1), cmul(hyz, a2));
+          yo[2 * N] = add_id<T>(xi[2 * N], cmul(hxz, a0), cmul(hyz, a1), cmul(hzz, a2));
         } else {  // 2: H u alone
           yo[0] = from_v<T>(cmul(hxx, a0) + cmul(hxy, a1) + cmul(hxz, a2));
           yo[N] = from_v<T>(cmul(hxy, a0) + cmul(hyy, a1) + cmul(hyz, a2));
