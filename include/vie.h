@@ -146,7 +146,8 @@ typedef struct {
  *          such nk > n (a circular convolution of length M >= 2n - 1 equals the
  *          zero-padded one on the n^3 nodes; n = 326 runs on M = 660).
  *          Register-resident kernels for M = 2n in {64, 96, 128, 192, 256, 384,
- *          512}, shared-memory Stockham kernels for the other grids.  The
+ *          512}, shared-memory kernels (two-step where M splits into two codelet
+ *          radices, else Stockham) for the other grids.  The
  *          oversampled set-up grid is 3n; when 3n has a prime factor above 11
  *          its lines are transformed by Bluestein's chirp-z algorithm over a
  *          padded length Q >= 2 (3n) - 1 made of the factors 2, 3, 5, 7, 11.
@@ -253,7 +254,8 @@ vie_status vie_problem_destroy(vie_problem* P);
  * applicable variant on this device; the choice is kept in the handle and
  * written to *variant (-1: the shape uses the generic kernels).  Variants:
  * 0/1/2 one CTA per mirror group of tiles with 8/16/4 pencils per tile, one
- * component per thread; 3 one CTA per tile of 8 pencils; 4/5/6 (FP32 only,
+ * component per thread; 3 one CTA per tile of 8 pencils (FP64: of 4, two-step
+ * transforms in place, where 2n splits); 4/5/6 (FP32 only,
  * 2n in {64, 96, 128, 256}) as 0/1/2 with two neighbouring pencils per
  * thread packed as f32x2 lanes; 7/8/9 (FP32 only, same sizes) mirror-group
  * CTAs of 8/4/16 pencils with all three components of a vector per thread;

@@ -8,9 +8,10 @@
 // on the n^3 output nodes; n = 326, 2n = 4 x 163, runs on M = 660).
 // Five passes over HBM.  For M = 2n in {64, 96, 128, 192, 256, 384, 512} they
 // are the register-resident kernels of apply_fast.cuh (chosen here, with the
-// z-pass autotuner); every other grid, and the double-word passes without a
-// fast kernel, run the shared-memory Stockham kernels of this file
-// (vie_fft.cuh):
+// z-pass autotuner); other grids, the double-word passes without a fast kernel
+// and some FP64 passes run the two-step kernels of vie_two.cuh where M = R1 R2
+// has a split into their radices, and the shared-memory Stockham kernels of this
+// file (vie_fft.cuh) where it has none:
 //   P1  x-lines: zero-pad n -> M, forward FFT           x [c][n][n][n]    -> A [c][n][n][M]
 //   P2  y-lines: zero-pad, forward FFT                   A                 -> B [c][n][M][M]
 //   P3  z-pencils of all components: zero-pad, forward FFT, per-k kernel
@@ -31,7 +32,7 @@
 #include "apply_fast.cuh"
 
 namespace vie {
-// Generic kernels (any line plan): shared-memory Stockham passes with the
+// Kernels of any line plan: shared-memory Stockham passes with the
 // twiddle table staged in shared memory (line_fft, vie_fft.cuh; the apply's
 // plans are direct, Bluestein's algorithm is taken by the set-up's 3n lines).
 // Tile lines have the plan's inner length Q (= M for a direct plan) plus one.
@@ -404,6 +405,23 @@ vie_status ensure_apply_workspace(vie_problem* P, const KernelSet& K, int prec, 
   return VIE_OK;
 }
 
+// The two-step passes in the arithmetic of T: radices up to 16 in kernels of
+// their own, which need fewer registers.
+template <typename T>
+static vie_status two_dispatch(int pass, const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
+  const bool small = p.R1 <= 16;
+  if (Prec<T>::id == VIE_FP32) return small ? two_pass_f32_16(pass, p, a, st) : two_pass_f32_24(pass, p, a, st);
+  if (Prec<T>::id == VIE_FP64) return small ? two_pass_f64_16(pass, p, a, st) : two_pass_f64_24(pass, p, a, st);
+  return small ? two_pass_df_16(pass, p, a, st) : two_pass_df_24(pass, p, a, st);
+}
+// Pass k of run_apply_t on its two-step plan.
+#define VIE_TWO(k)                                            \
+  do {                                                        \
+    vie_status e_ = two_dispatch<T>(k, tp, ta, st);           \
+    if (e_ != VIE_OK) return e_;                              \
+    if (rec) VIE_CK(cudaEventRecord(ev[k], st));              \
+  } while (0)
+
 template <typename T>
 static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in, void* out, int nrhs,
                               int with_identity, cudaStream_t st) {
@@ -433,13 +451,11 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     ++pf.count;
   }
 
-  // double-word arithmetic runs on the generic kernels only: its fully
-  // unrolled register-resident variants take far too long to compile
   FastSel fs = fast_select(fast_grid(P), K.mode, with_identity);
   if (Prec<T>::id == VIE_DF64) {
     // double-word fast kernels exist for 2n = 256 and the operator's kernel sets
-    // only; its register-resident P5 (254 registers, one CTA per SM) is slower
-    // than the generic one, which it keeps
+    // only (z pass 1.19 ms, two-step 1.34); its register-resident P5 (254
+    // registers, one CTA per SM) is slower than the two-step one (0.32 ms)
     if (!(M == 256 && fs.p1 && (K.mode == KM_SYM3 || K.mode == KM_MAXWELL6))) fs = FastSel();
     fs.p5 = false;
   }
@@ -466,11 +482,21 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     }
   }
   if (p3v == kP3Generic) fs.p3 = false;
+  TwoPlan tp;
+  const bool two = make_two_plan(M, &tp);
+  if (Prec<T>::id == VIE_FP64 && fp64_two_y(M)) {
+    fs.py = false;
+    if (fp64_two_last(M)) fs.p5 = false;
+  }
+  TwoArgs ta = {n, K.mode, C, cin, cout, nrhs, with_identity, in, Prec<T>::He(P), P->has_mu ? Prec<T>::Hm(P) : nullptr,
+                Kp, tw, out, A, B};
   // P1
   if (fs.p1) {
     vie_status e = fast_dispatch(1, P, K, in, out, nrhs, with_identity, A, B, C, Prec<T>::id, st);
     if (e != VIE_OK) return e;
     if (rec) VIE_CK(cudaEventRecord(ev[1], st));
+  } else if (two) {
+    VIE_TWO(1);
   } else {
     const int nl = lines_for(pl, vs);
     const size_t smem = tile_smem(pl, vs, nl);
@@ -487,6 +513,8 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     vie_status e = fast_dispatch(2, P, K, in, out, nrhs, with_identity, A, B, C, Prec<T>::id, st);
     if (e != VIE_OK) return e;
     if (rec) VIE_CK(cudaEventRecord(ev[2], st));
+  } else if (two) {
+    VIE_TWO(2);
   } else {
     VIE_CK(allow_smem(k_py<T, -1>));
     dim3 grid(M / nly, n, nrhs * cin);
@@ -502,7 +530,9 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     if (!used) fs.p3 = false;  // no fast z pass fits this shape: the generic one below
     else if (rec) VIE_CK(cudaEventRecord(ev[3], st));
   }
-  if (!fs.p3) {
+  if (!fs.p3 && two && two_z_fits(tp, Prec<T>::id == VIE_DF64)) {
+    VIE_TWO(3);
+  } else if (!fs.p3) {
     int nl = pow2_divisor(M, 8);
     // two CTAs per SM: the z pass is compute bound and needs the warps
     while (nl > 1 && tile_smem(pl, vs, C * nl) > 110 * 1024) nl >>= 1;
@@ -518,6 +548,8 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     vie_status e = fast_dispatch(4, P, K, in, out, nrhs, with_identity, A, B, C, Prec<T>::id, st);
     if (e != VIE_OK) return e;
     if (rec) VIE_CK(cudaEventRecord(ev[4], st));
+  } else if (two) {
+    VIE_TWO(4);
   } else {
     VIE_CK(allow_smem(k_py<T, +1>));
     dim3 grid(M / nly, n, nrhs * cout);
@@ -530,6 +562,8 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
     vie_status e = fast_dispatch(5, P, K, in, out, nrhs, with_identity, A, B, C, Prec<T>::id, st);
     if (e != VIE_OK) return e;
     if (rec) VIE_CK(cudaEventRecord(ev[5], st));
+  } else if (two) {
+    VIE_TWO(5);
   } else {
     int nr = 4;
     while (nr > 1 && tile_smem(pl, vs, cout * nr) > 200 * 1024) nr >>= 1;

@@ -10,6 +10,7 @@
 
 #include "vie_fft2.cuh"
 #include "vie_internal.h"
+#include "vie_two.cuh"
 
 namespace vie {
 
@@ -1428,6 +1429,14 @@ __global__ void __launch_bounds__(256) f_p5(const typename CT<T>::V* __restrict_
 
 inline size_t smem_optin() { return (size_t)smem_optin_bytes(); }
 
+// FP64 passes of the fast grids that run the two-step kernels (vie_two.cuh): the
+// y passes up to M = 256, where both their radices are at most 16 (64^3: 122 and
+// 125 us against 133 and 140), and the last pass up to M = 96 (32^3: 23 us
+// against 49, whose 8-point lines keep one CTA an SM; from 64^3 on f_p5 is ahead,
+// 105 us against 123).  The z pass is the tuner's choice (p3_tile).
+constexpr bool fp64_two_y(int M) { return M == 64 || M == 96 || M == 128 || M == 192 || M == 256; }
+constexpr bool fp64_two_last(int M) { return M == 64 || M == 96; }
+
 // Fast-path launches for 2n = R1 R2; returns false if a pass must use the generic kernels.
 template <typename T, int R1, int R2>
 struct FastPath {
@@ -1444,10 +1453,14 @@ struct FastPath {
   }
   template <int S>
   static vie_status py(const V* in, V* out, int n, int C, int nc, int nrhs, const V* tw, cudaStream_t st) {
-    VIE_CK(allow_smem(f_py<T, R1, R2, S>));
-    f_py<T, R1, R2, S><<<dim3(M / L, n, nrhs * nc), 256, smem(), st>>>(in, out, n, C, nc, tw);
-    VIE_CK(cudaGetLastError());
-    return VIE_OK;
+    if constexpr (std::is_same<T, double>::value && fp64_two_y(M)) {
+      return VIE_EINVAL;  // not dispatched here
+    } else {
+      VIE_CK(allow_smem(f_py<T, R1, R2, S>));
+      f_py<T, R1, R2, S><<<dim3(M / L, n, nrhs * nc), 256, smem(), st>>>(in, out, n, C, nc, tw);
+      VIE_CK(cudaGetLastError());
+      return VIE_OK;
+    }
   }
   template <int MODE, int NP>
   static vie_status p3b(V* B, int n, int C, const V* K, int nrhs, const V* tw, cudaStream_t st) {
@@ -1619,6 +1632,23 @@ struct FastPath {
       return e;
     }
   }
+  // Variant 3, one CTA per tile.  FP64 takes the two-step kernel (tiles of 4
+  // pencils, transforms in place) where 2n splits: the tuner weighs it against the
+  // mirror-group kernels.  z pass at 64^3, two-step against the best of those:
+  // Helmholtz 642 and 687 us, E and H of reduced Maxwell 963 and 1128 us.
+  template <int MODE>
+  static vie_status p3_tile(V* B, int n, int C, const V* K, int nrhs, const V* tw, bool* done, cudaStream_t st) {
+    if constexpr (std::is_same<T, double>::value) {
+      TwoPlan tp;
+      if (make_two_plan(M, &tp)) {
+        const TwoArgs a = {n, MODE, C, 0, 0, nrhs, 0, nullptr, nullptr, nullptr, K, tw, nullptr, nullptr, B};
+        vie_status e = tp.R1 <= 16 ? two_pass_f64_16(3, tp, a, st) : two_pass_f64_24(3, tp, a, st);
+        *done = e == VIE_OK;
+        return e;
+      }
+    }
+    return p3b_ok<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
+  }
   template <int MODE>
   static vie_status p3_mode(int variant, V* B, int n, int C, const V* K, int nrhs, const V* tw, bool* done,
                             cudaStream_t st) {
@@ -1626,7 +1656,7 @@ struct FastPath {
       case 0: return p3c<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
       case 1: return p3c<MODE, 16>(B, n, C, K, nrhs, tw, done, st);
       case 2: return p3c<MODE, 4>(B, n, C, K, nrhs, tw, done, st);
-      case 3: return p3b_ok<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
+      case 3: return p3_tile<MODE>(B, n, C, K, nrhs, tw, done, st);
       case 4: return p3p<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
       case 5: return p3p<MODE, 16>(B, n, C, K, nrhs, tw, done, st);
       case 6: return p3p<MODE, 4>(B, n, C, K, nrhs, tw, done, st);
@@ -1647,25 +1677,30 @@ struct FastPath {
   // Run P3 variant `variant` (0..kP3Variants-1); *done = false if it does not apply to this shape.
   static vie_status p3v(int variant, V* B, int n, int C, const V* K, int mode, int nrhs, const V* tw, bool* done,
                         cudaStream_t st) {
-    switch (mode) {
-      case KM_SYM3: return p3_mode<KM_SYM3>(variant, B, n, C, K, nrhs, tw, done, st);
-      case KM_DIV: return p3_mode<KM_DIV>(variant, B, n, C, K, nrhs, tw, done, st);
-      case KM_EMRED: return p3_mode<KM_EMRED>(variant, B, n, C, K, nrhs, tw, done, st);
-      default: return p3_mode<KM_MAXWELL6>(variant, B, n, C, K, nrhs, tw, done, st);
-    }
+    if (mode == KM_SYM3) return p3_mode<KM_SYM3>(variant, B, n, C, K, nrhs, tw, done, st);
+    if (mode == KM_MAXWELL6) return p3_mode<KM_MAXWELL6>(variant, B, n, C, K, nrhs, tw, done, st);
+    if constexpr (std::is_same<T, double>::value)  // the scattered field's kernel sets are FP64 only
+      return mode == KM_DIV ? p3_mode<KM_DIV>(variant, B, n, C, K, nrhs, tw, done, st)
+                            : p3_mode<KM_EMRED>(variant, B, n, C, K, nrhs, tw, done, st);
+    set_error("the scattered field is evaluated in FP64");
+    return VIE_EINVAL;
   }
   static vie_status p5(const V* A, const E* xin, E* y, int n, int C, int cout, const V* He, const V* Hm, int wid,
                        int nrhs, const V* tw, cudaStream_t st) {
     const dim3 grid((n * n + L - 1) / L, nrhs);
-    if (cout <= 3) {
-      VIE_CK(allow_smem(f_p5<T, R1, R2, 3>));
-      f_p5<T, R1, R2, 3><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+    if constexpr (std::is_same<T, df>::value || (std::is_same<T, double>::value && fp64_two_last(M))) {
+      return VIE_EINVAL;  // not dispatched here
     } else {
-      VIE_CK(allow_smem(f_p5<T, R1, R2, 6>));
-      f_p5<T, R1, R2, 6><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+      if (cout <= 3) {
+        VIE_CK(allow_smem(f_p5<T, R1, R2, 3>));
+        f_p5<T, R1, R2, 3><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+      } else {
+        VIE_CK(allow_smem(f_p5<T, R1, R2, 6>));
+        f_p5<T, R1, R2, 6><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+      }
+      VIE_CK(cudaGetLastError());
+      return VIE_OK;
     }
-    VIE_CK(cudaGetLastError());
-    return VIE_OK;
   }
 };
 
@@ -1773,7 +1808,7 @@ vie_status tune_p3(vie_problem* P, const KernelSet& K, typename CT<T>::V* B, int
 // Maxwell 6x6), one fixed schedule each (8 pencils per tile, 4 for Maxwell),
 // no tuning.  Instantiated for 2n = 256 only, in its own translation unit
 // (apply_fast_dw_256.cu): the unrolled double-word codelets are long to
-// compile, so every other shape and mode keeps the generic kernels.
+// compile, so every other shape and mode runs the two-step kernels.
 // *used = false if this (pass, mode) has no double-word fast kernel.
 template <int R1, int R2>
 vie_status fast_pass_dw(int pass, vie_problem* P, const KernelSet& K, const void* in, void* out, int nrhs,

@@ -1,0 +1,8 @@
+// Two-step passes of the apply, FP32, first radix up to 16 (see vie_two.cuh).
+#include "vie_two.cuh"
+
+namespace vie {
+vie_status two_pass_f32_16(int pass, const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
+  return two_pass<float, 16>(pass, p, a, st);
+}
+}  // namespace vie

@@ -552,6 +552,76 @@ template <int S, typename T> struct Dft<5, S, T> : DftOdd<5, S, T> {};
 template <int S, typename T> struct Dft<7, S, T> : DftOdd<7, S, T> {};
 template <int S, typename T> struct Dft<11, S, T> : DftOdd<11, S, T> {};
 
+// DFT of length P Q, P and Q coprime, by the prime-factor split (Good 1958, Thomas
+// 1963): with n = Q n1 + P n2 and k = (Q Q^-1) k1 + (P P^-1) k2 modulo P Q the
+// twiddles between the two steps are all 1.
+template <int P, int Q, int S, typename T>
+struct DftPFA {
+  typedef typename CT<T>::V V;
+  static constexpr int inverse(int a, int m) {
+    int x = 1;
+    while ((a * x) % m != 1 % m) ++x;
+    return x;
+  }
+  static __device__ __forceinline__ void run(V* u) {
+    constexpr int N = P * Q, A = Q * inverse(Q % P, P), B = P * inverse(P % Q, Q);
+    V y[P][Q];
+#pragma unroll
+    for (int n2 = 0; n2 < Q; ++n2) {
+      V t[P];
+#pragma unroll
+      for (int n1 = 0; n1 < P; ++n1) t[n1] = u[(Q * n1 + P * n2) % N];
+      Dft<P, S, T>::run(t);
+#pragma unroll
+      for (int k1 = 0; k1 < P; ++k1) y[k1][n2] = t[k1];
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < P; ++k1) {
+      Dft<Q, S, T>::run(y[k1]);
+#pragma unroll
+      for (int k2 = 0; k2 < Q; ++k2) u[(A * k1 + B * k2) % N] = y[k1][k2];
+    }
+  }
+};
+
+// n = 3 n1 + n2, k = k1 + 3 k2 with the four twiddles exp(S 2 pi i n2 k1 / 9).
+template <int S, typename T> struct Dft<9, S, T> {
+  typedef typename CT<T>::V V;
+  static __device__ __forceinline__ void run(V* u) {
+    const double c[5] = {1.0, 0.76604444311897803520, 0.17364817766693034885, -0.5, -0.93969262078590838405};
+    const double s[5] = {0.0, 0.64278760968653932632, 0.98480775301220805937, 0.86602540378443864676,
+                         0.34202014332566873304};
+    V y[3][3];
+#pragma unroll
+    for (int n2 = 0; n2 < 3; ++n2) {
+      V t[3] = {u[n2], u[3 + n2], u[6 + n2]};
+      Dft<3, S, T>::run(t);
+#pragma unroll
+      for (int k1 = 0; k1 < 3; ++k1) {
+        const int j = n2 * k1;
+        y[k1][n2] = j == 0 ? t[k1] : rot(t[k1], (T)c[j], (T)(S * s[j]));
+      }
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      Dft<3, S, T>::run(y[k1]);
+#pragma unroll
+      for (int k2 = 0; k2 < 3; ++k2) u[k1 + 3 * k2] = y[k1][k2];
+    }
+  }
+};
+
+template <int S, typename T> struct Dft<6, S, T> : DftPFA<2, 3, S, T> {};
+template <int S, typename T> struct Dft<10, S, T> : DftPFA<2, 5, S, T> {};
+template <int S, typename T> struct Dft<12, S, T> : DftPFA<4, 3, S, T> {};
+template <int S, typename T> struct Dft<14, S, T> : DftPFA<2, 7, S, T> {};
+template <int S, typename T> struct Dft<15, S, T> : DftPFA<3, 5, S, T> {};
+template <int S, typename T> struct Dft<18, S, T> : DftPFA<2, 9, S, T> {};
+template <int S, typename T> struct Dft<20, S, T> : DftPFA<4, 5, S, T> {};
+template <int S, typename T> struct Dft<21, S, T> : DftPFA<3, 7, S, T> {};
+template <int S, typename T> struct Dft<22, S, T> : DftPFA<2, 11, S, T> {};
+template <int S, typename T> struct Dft<24, S, T> : DftPFA<8, 3, S, T> {};
+
 // ------------------------------------------------------------ FFT plan
 // A line DFT of length M runs as radix stages of length Q.  Q = M when M
 // factors into the codelet radices; otherwise Q is the smallest such length

@@ -110,37 +110,6 @@ __device__ __forceinline__ typename CT<T>::V twc(typename CT<T>::V a, int j) {
   return rot(a, (T)c, (T)s);
 }
 
-// DFT of length P Q on registers by the same two-step split as the line FFT:
-// X[k1 + P k2] = sum_{n2} W_Q^{n2 k2} W_{PQ}^{n2 k1} sum_{n1} W_P^{n1 k1} x[Q n1 + n2].
-template <int P, int Q, int S, typename T>
-struct DftPQ {
-  typedef typename CT<T>::V V;
-  static __device__ __forceinline__ void run(V* u) {
-    V y[Q][P];
-#pragma unroll
-    for (int n2 = 0; n2 < Q; ++n2) {
-#pragma unroll
-      for (int n1 = 0; n1 < P; ++n1) y[n2][n1] = u[Q * n1 + n2];
-      Dft<P, S, T>::run(y[n2]);
-#pragma unroll
-      for (int k1 = 1; k1 < P; ++k1)
-        if (n2 != 0) y[n2][k1] = twc<P * Q, S, T>(y[n2][k1], n2 * k1);
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < P; ++k1) {
-      V z[Q];
-#pragma unroll
-      for (int n2 = 0; n2 < Q; ++n2) z[n2] = y[n2][k1];
-      Dft<Q, S, T>::run(z);
-#pragma unroll
-      for (int k2 = 0; k2 < Q; ++k2) u[k1 + P * k2] = z[k2];
-    }
-  }
-};
-template <int S, typename T> struct Dft<6, S, T> : DftPQ<2, 3, S, T> {};
-template <int S, typename T> struct Dft<12, S, T> : DftPQ<4, 3, S, T> {};
-template <int S, typename T> struct Dft<24, S, T> : DftPQ<8, 3, S, T> {};
-
 template <int S, typename T> struct Dft<32, S, T> {
   typedef typename CT<T>::V V;
   static __device__ __forceinline__ void run(V* u) {
