@@ -18,6 +18,7 @@
 #include <chrono>
 #include <cmath>
 #include <complex>
+#include <type_traits>
 #include <vector>
 
 #include "vie_internal.h"
@@ -285,6 +286,7 @@ struct ArnState {
   double wn2;    // |w|^2 of the current step before projection
   double beta;   // initial residual norm of the cycle
   double ynorm;  // |y| of the cycle's least-squares solution: the norm of its correction
+  int exp2;      // the current step's vector is stored with norm in [1/2, 1) times 2^exp2
 };
 
 __host__ __device__ __forceinline__ double2 dconj(double2 a) { return make_double2(a.x, -a.y); }
@@ -302,7 +304,7 @@ struct ArnLayout {
   double2* sn = nullptr;       // [nb][m]
   double2* gv = nullptr;       // [nb][m + 1] rotated right-hand side of the least squares
   double2* hcol = nullptr;     // [nb][2][m + 2] coefficients of passes 0 and 1
-  double2* coef = nullptr;     // [nb][m] update coefficients y_i s_i
+  double2* coef = nullptr;     // [nb][m] projection coefficients of a pass; at the end y_i s_i
   double2* partial = nullptr;  // [nb][m + 3][G] block partial sums
   unsigned* cnt = nullptr;     // [nb] last-block counters
 };
@@ -355,18 +357,73 @@ template <> struct Pack<double2> {
   static __device__ __forceinline__ void put(double2& p, int, double2 v) { p = v; }
 };
 
-// Pass p: block partials of <W_i, W_{j+1}>, i <= j (pass 0 also |W_{j+1}|^2); the last
-// block stores h_i = s_i s_j <W_i, W_{j+1}> and (pass 0) |w|^2 = s_j^2 |W_{j+1}|^2.
-// Vectors are read in 16-byte packs, two packs in flight per thread; ldi and L
-// are multiples of the pack width except for an odd tail handled element-wise.
+// Block partials of CNT inner products <W_i, w>, i = i0 .. i0 + CNT - 1, over units of
+// U values (16-byte packs where aligned, else single values); SELF: also |w|^2.
+// CNT is a compile-time constant so that a unit's CNT + 1 loads are all issued
+// before the first is used (a run-time count puts a branch before each).
+template <typename TB, typename U, int CNT, bool SELF>
+__device__ __forceinline__ void arn_chunk(const TB* V, long long ldi, const TB* w, long long units,
+                                          typename Acc<TB>::T* ar, typename Acc<TB>::T* ai) {
+  constexpr int W = sizeof(U) / sizeof(TB);
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  typename Acc<TB>::T br[CNT + 1], bi[CNT + 1];  // sums of every other unit
+#pragma unroll
+  for (int t = 0; t < CNT + 1; ++t) ar[t] = ai[t] = br[t] = bi[t] = 0;
+  auto add = [&](const U& y, const U* x, typename Acc<TB>::T* sr, typename Acc<TB>::T* si) {
+#pragma unroll
+    for (int q = 0; q < W; ++q) {
+      const TB c = ((const TB*)&y)[q];
+#pragma unroll
+      for (int t = 0; t < CNT; ++t) {
+        const TB v = ((const TB*)&x[t])[q];
+        sr[t] += v.x * c.x + v.y * c.y;
+        si[t] += v.x * c.y - v.y * c.x;
+      }
+      if (SELF) sr[CNT] += c.x * c.x + c.y * c.y;
+    }
+  };
+  long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (; e + stride < units; e += 2 * stride) {
+    U x[CNT], z[CNT];
+    const U y = ((const U*)w)[e], y2 = ((const U*)w)[e + stride];
+#pragma unroll
+    for (int t = 0; t < CNT; ++t) {
+      x[t] = ((const U*)(V + t * ldi))[e];
+      z[t] = ((const U*)(V + t * ldi))[e + stride];
+    }
+    add(y, x, ar, ai);
+    add(y2, z, br, bi);
+  }
+  if (e < units) {
+    U x[CNT];
+    const U y = ((const U*)w)[e];
+#pragma unroll
+    for (int t = 0; t < CNT; ++t) x[t] = ((const U*)(V + t * ldi))[e];
+    add(y, x, ar, ai);
+  }
+#pragma unroll
+  for (int t = 0; t < CNT + (SELF ? 1 : 0); ++t) {
+    ar[t] += br[t];
+    ai[t] += bi[t];
+  }
+}
+
+// Pass p: block partials of <W_i, W_{j+1}>, i <= j (pass 0 also |W_{j+1}|^2, in slot
+// j + 1); the last block stores h_i = s_i s_j <W_i, W_{j+1}>, the coefficients h_i s_i /
+// s_{j+1} of the projection in the basis precision, and (pass 0) |w|^2 = s_j^2
+// |W_{j+1}|^2 with the power of two of the projection (k_arn_axpy), so that the
+// blocks of k_arn_axpy start without FP64 divisions and roots of their own (the
+// FP64 unit takes a warp instruction in 16 cycles).
+// Bound by HBM at large grids: Helmholtz 128^3, seven basis vectors on average,
+// 120 -> 88 us a step (4.9 TB/s); Maxwell 64^3 with eight right-hand sides, 37 steps
+// 11.5 -> 8.4 ms.
 template <typename TB>
 __global__ void __launch_bounds__(kRedThreads) k_arn_dots(const TB* __restrict__ V, long long ldi, int j, long long L,
                                                           ArnLayout A, int pass) {
   typedef typename Acc<TB>::T AT;
-  typedef Pack<TB> PK;
-  typedef typename PK::P P;
-  constexpr int W = PK::W;
-  __shared__ double2 red[kRedThreads / 32][kDotChunk];
+  typedef typename Pack<TB>::P P;
+  constexpr int W = Pack<TB>::W;
+  __shared__ double2 red[kRedThreads / 32][kDotChunk + 1];
   const int r = blockIdx.y, G = gridDim.x, m = A.m, ldp = m + 3;
   ArnState* S = A.st + r;
   if (S->done || (pass == 1 && !S->reorth)) return;  // block-uniform
@@ -374,75 +431,49 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_dots(const TB* __restrict__
   const TB* wr = V + (long long)(j + 1) * ldi + (long long)r * L;
   const int k = j + 1, ktot = k + (pass == 0 ? 1 : 0);
   // packs when every vector start is pack-aligned (ldi, L multiples of W), else element-wise
-  const bool packed = (W > 1) && (ldi % W == 0) && (L % W == 0);
-  const long long NP = packed ? L / W : 0;  // packs per vector
-  const long long stride = (long long)G * blockDim.x;
-  const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  for (int i0 = 0; i0 < ktot; i0 += kDotChunk) {
-    const int cnt = min(kDotChunk, ktot - i0);
-    AT ar[kDotChunk], ai[kDotChunk];
-#pragma unroll
-    for (int t = 0; t < kDotChunk; ++t) ar[t] = ai[t] = (AT)0;
-    auto acc1 = [&](int t, TB v, TB we) {
-      ar[t] += v.x * we.x + v.y * we.y;
-      ai[t] += v.x * we.y - v.y * we.x;
-    };
-    if (packed) {
-      const P* wp = (const P*)wr;
-      long long e = tid;
-      for (; e + stride < NP; e += 2 * stride) {
-        const P wa = wp[e], wb = wp[e + stride];
-#pragma unroll
-        for (int t = 0; t < kDotChunk; ++t)
-          if (t < cnt) {
-            const int i = i0 + t;
-            const P va = (i < k) ? ((const P*)(Vr + (long long)i * ldi))[e] : wa;
-            const P vb = (i < k) ? ((const P*)(Vr + (long long)i * ldi))[e + stride] : wb;
-#pragma unroll
-            for (int q = 0; q < W; ++q) {
-              acc1(t, PK::get(va, q), PK::get(wa, q));
-              acc1(t, PK::get(vb, q), PK::get(wb, q));
-            }
-          }
+  const bool packed = (W == 1) || ((ldi % W == 0) && (L % W == 0));
+  for (int i0 = 0; i0 < k; i0 += kDotChunk) {
+    const int cnt = min(kDotChunk, k - i0);
+    const bool self = pass == 0 && i0 == 0;
+    AT ar[kDotChunk + 1], ai[kDotChunk + 1];
+    const TB* Vi = Vr + (long long)i0 * ldi;
+    auto go = [&](auto cc) {
+      constexpr int C = decltype(cc)::value;
+      if (packed) {
+        if (self) arn_chunk<TB, P, C, true>(Vi, ldi, wr, L / W, ar, ai);
+        else arn_chunk<TB, P, C, false>(Vi, ldi, wr, L / W, ar, ai);
+      } else {
+        if (self) arn_chunk<TB, TB, C, true>(Vi, ldi, wr, L, ar, ai);
+        else arn_chunk<TB, TB, C, false>(Vi, ldi, wr, L, ar, ai);
       }
-      for (; e < NP; e += stride) {
-        const P wa = wp[e];
+      // warp sums in the accumulation type, cross-warp in FP64
 #pragma unroll
-        for (int t = 0; t < kDotChunk; ++t)
-          if (t < cnt) {
-            const int i = i0 + t;
-            const P va = (i < k) ? ((const P*)(Vr + (long long)i * ldi))[e] : wa;
-#pragma unroll
-            for (int q = 0; q < W; ++q) acc1(t, PK::get(va, q), PK::get(wa, q));
+      for (int t = 0; t < C + 1; ++t)
+        if (t < C || self) {
+          AT ax = ar[t], ay = ai[t];
+          for (int off = 16; off > 0; off >>= 1) {
+            ax += __shfl_down_sync(0xffffffffu, ax, off);
+            ay += __shfl_down_sync(0xffffffffu, ay, off);
           }
-      }
-    } else {
-      for (long long e = tid; e < L; e += stride) {
-        const TB we = wr[e];
-#pragma unroll
-        for (int t = 0; t < kDotChunk; ++t)
-          if (t < cnt) {
-            const int i = i0 + t;
-            acc1(t, (i < k) ? Vr[(long long)i * ldi + e] : we, we);
-          }
-      }
-    }
-    // warp sums in the accumulation type (slots in use only), cross-warp in FP64
-#pragma unroll
-    for (int t = 0; t < kDotChunk; ++t)
-      if (t < cnt) {
-        AT ax = ar[t], ay = ai[t];
-        for (int off = 16; off > 0; off >>= 1) {
-          ax += __shfl_down_sync(0xffffffffu, ax, off);
-          ay += __shfl_down_sync(0xffffffffu, ay, off);
+          if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][t] = make_double2((double)ax, (double)ay);
         }
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][t] = make_double2((double)ax, (double)ay);
-      }
+    };
+    switch (cnt) {
+      case 1: go(std::integral_constant<int, 1>{}); break;
+      case 2: go(std::integral_constant<int, 2>{}); break;
+      case 3: go(std::integral_constant<int, 3>{}); break;
+      case 4: go(std::integral_constant<int, 4>{}); break;
+      case 5: go(std::integral_constant<int, 5>{}); break;
+      case 6: go(std::integral_constant<int, 6>{}); break;
+      case 7: go(std::integral_constant<int, 7>{}); break;
+      default: go(std::integral_constant<int, 8>{}); break;
+    }
     __syncthreads();
-    if (threadIdx.x < cnt) {
+    if (threadIdx.x < cnt + (self ? 1 : 0)) {
       double2 sm = make_double2(0, 0);
       for (int w = 0; w < kRedThreads / 32; ++w) sm = sm + red[w][threadIdx.x];
-      A.partial[((long long)r * ldp + i0 + threadIdx.x) * G + blockIdx.x] = sm;
+      const int slot = threadIdx.x < cnt ? i0 + threadIdx.x : k;
+      A.partial[((long long)r * ldp + slot) * G + blockIdx.x] = sm;
     }
     __syncthreads();
   }
@@ -451,23 +482,36 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_dots(const TB* __restrict__
   if (threadIdx.x == 0) A.cnt[r] = 0;
   const double* sc = A.sc + (long long)r * (m + 2);
   double2* h = A.hcol + ((long long)r * 2 + pass) * (m + 2);
+  typename Acc<TB>::V* cf = (typename Acc<TB>::V*)(A.coef + (long long)r * m);
   const double sj = sc[j + 1];  // scale of W_{j+1} as currently stored
   for (int i = threadIdx.x; i < ktot; i += blockDim.x) {
     const double2 raw = A.partial[((long long)r * ldp + i) * G];
-    if (i < k) h[i] = dscale(sc[i] * sj, raw);
-    else S->wn2 = sj * sj * raw.x;
+    if (i < k) {
+      const double si = sc[i];
+      const double2 hi = dscale(si * sj, raw);
+      h[i] = hi;
+      const double f = si / sj;
+      cf[i].x = (AT)(hi.x * f);
+      cf[i].y = (AT)(hi.y * f);
+    } else {
+      S->wn2 = sj * sj * raw.x;
+      // E with |W_{j+1}| = f 2^E, f in [1/2, 1), clamped so that 2^-E stays a normal FP32 number
+      const double rawn = sqrt(raw.x);
+      int E = 0;
+      if (rawn > 0.0 && isfinite(rawn)) frexp(rawn, &E);
+      S->exp2 = E < -100 ? -100 : (E > 100 ? 100 : E);
+    }
   }
 }
 
 // Finalise step j of member r (called by the whole block, thread 0 does the
 // serial part): Hessenberg column h (i <= j) and h_{j+1,j} = hn; rotations,
 // residual estimate, next scale, done flag.  The column and the earlier
-// rotations are staged in shared memory by all threads first, so that the
-// serial rotation chain runs on shared memory instead of making a dependent
-// global-memory round trip per rotation.
+// rotations are staged in shared memory by all threads first.
 static const int kMaxRestart = 200;
 __device__ void arn_finalize(ArnLayout& A, int r, int j, const double2* h0, const double2* h1, double hn) {
-  __shared__ double2 col[kMaxRestart + 1], csh[kMaxRestart], snh[kMaxRestart];
+  __shared__ double2 col[kMaxRestart + 1], csh[kMaxRestart], tsh[kMaxRestart + 1];
+  __shared__ double snh[kMaxRestart];
   __shared__ int bad;
   const int m = A.m;
   ArnState* S = A.st + r;
@@ -486,29 +530,44 @@ __device__ void arn_finalize(ArnLayout& A, int r, int j, const double2* h0, cons
     col[i] = v;
     if (i < j) {
       csh[i] = cs[i];
-      snh[i] = sn[i];
+      snh[i] = sn[i].x;
     }
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
   if (bad) {
-    S->nan = 1;
-    S->done = 1;
+    if (threadIdx.x == 0) {
+      S->nan = 1;
+      S->done = 1;
+    }
     return;
   }
-  // earlier rotations G_i = [[conj(c_i), conj(s_i)], [-s_i, c_i]] on rows i, i+1
-  double2 a = col[0];
-  for (int i = 0; i < j; ++i) {
-    const double2 b = col[i + 1];
-    col[i] = cmul(dconj(csh[i]), a) + cmul(dconj(snh[i]), b);
-    a = cmul(csh[i], b) - cmul(snh[i], a);
+  // earlier rotations G_i = [[conj(c_i), s_i], [-s_i, c_i]] (s_i real) on rows i, i+1:
+  // a_0 = col_0, a_{i+1} = c_i col_{i+1} - s_i a_i, and R_i = conj(c_i) a_i + s_i
+  // col_{i+1}.  Only a_{i+1} = t_i - s_i a_i is a chain, one FMA a step on each of two
+  // lanes; the products t_i and the R_i are formed by all threads.
+  for (int i = threadIdx.x; i < j; i += blockDim.x) tsh[i] = cmul(csh[i], col[i + 1]);
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double x = ((const double*)&col[0])[threadIdx.x];
+    for (int i = 0; i < j; ++i) {
+      const double t = ((const double*)&tsh[i])[threadIdx.x];
+      ((double*)&tsh[i])[threadIdx.x] = x;  // a_i in place of t_i
+      x = fma(-snh[i], x, t);
+    }
+    ((double*)&tsh[j])[threadIdx.x] = x;
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < j; i += blockDim.x) {
+    const double2 v = cmul(dconj(csh[i]), tsh[i]);
+    Rc[i] = make_double2(fma(snh[i], col[i + 1].x, v.x), fma(snh[i], col[i + 1].y, v.y));
+  }
+  if (threadIdx.x != 0) return;
+  const double2 a = tsh[j];
   const double den = sqrt(dnorm2(a) + hn * hn);
   const double id = den > 0 ? 1.0 / den : 0.0;
   const double2 c = den > 0 ? dscale(id, a) : make_double2(1, 0);
   const double2 sv = make_double2(hn * id, 0);
-  col[j] = cmul(dconj(c), a) + dscale(hn, dconj(sv));
-  for (int i = 0; i <= j; ++i) Rc[i] = col[i];
+  Rc[j] = cmul(dconj(c), a) + dscale(hn, dconj(sv));
   cs[j] = c;
   sn[j] = sv;
   const double2 gj = g[j];
@@ -534,7 +593,10 @@ __device__ void arn_finalize(ArnLayout& A, int r, int j, const double2* h0, cons
 // divides s_{j+1} by c: a power of two leaves every mantissa as it was, and the
 // stored basis stays near unit norm.  Without it each stored vector would be
 // about h_{j+1,j} times the previous one, which overflows the FP32 basis within
-// a cycle when the operator norm is large (tens, at high frequency).
+// a cycle when the operator norm is large (tens, at high frequency).  The
+// coefficients and c were left by k_arn_dots.  Laplace 32^3, 15 steps: 254 -> 185
+// us with those and the parallel rotations of arn_finalize (the FP64 unit's
+// latency was most of a short vector's step).
 template <typename TB>
 __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, long long ldi, int j, long long L,
                                                           ArnLayout A, int pass) {
@@ -545,23 +607,12 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
   ArnState* S = A.st + r;
   if (S->done || (pass == 1 && !S->reorth)) return;  // block-uniform
   double* sc = A.sc + (long long)r * (m + 2);
-  const double2* h = A.hcol + ((long long)r * 2 + pass) * (m + 2);
   const int k = j + 1;
-  const double u = sc[j + 1];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    const double f = sc[i] / u;
-    cf[i].x = (AT)(h[i].x * f);
-    cf[i].y = (AT)(h[i].y * f);
-  }
-  // c = 2^-E with |W_{j+1}| = f 2^E, f in [1/2, 1) (|W_{j+1}|^2 = wn2 / u^2), E clamped
-  // so that c stays a normal FP32 number
-  int E = 0;
-  if (pass == 0) {
-    const double rawn = sqrt(S->wn2) / u;
-    if (rawn > 0.0 && isfinite(rawn)) frexp(rawn, &E);
-    E = E < -100 ? -100 : (E > 100 ? 100 : E);
-  }
-  const AT cscale = (AT)ldexp(1.0, -E);
+  const typename Acc<TB>::V* cg = (const typename Acc<TB>::V*)(A.coef + (long long)r * m);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = cg[i];
+  // c = 2^-E
+  const int E = pass == 0 ? S->exp2 : 0;
+  const AT cscale = (AT)ldexpf(1.0f, -E);
   __syncthreads();
   const TB* Vr = V + (long long)r * L;
   TB* wr = V + (long long)(j + 1) * ldi + (long long)r * L;
@@ -569,7 +620,7 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
   typedef Pack<TB> PK;
   typedef typename PK::P P;
   constexpr int W = PK::W;
-  const bool packed = (W > 1) && (ldi % W == 0) && (L % W == 0);
+  const bool packed = (W == 1) || ((ldi % W == 0) && (L % W == 0));
   const long long NPK = packed ? L / W : L;  // units (packs or elements) per vector
   const long long stride = (long long)G * blockDim.x;
   // one unit: W elements of W_{j+1} at unit e, minus the projection, and its |.|^2
@@ -588,42 +639,41 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
     for (int q = 0; q < W; ++q)
 #pragma unroll
       for (int u = 0; u < 4; ++u) sx[q][u] = sy[q][u] = 0;
-    int i = 0;
-    for (; i + 4 <= k; i += 4) {  // four basis loads in flight
+    // N basis loads in flight, then their products into N / 2 (or 1) partial sums
+    auto terms = [&](int i, auto nc) {
+      constexpr int N = decltype(nc)::value;
+      if (packed) {
+        P pv[N];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const typename Acc<TB>::V c = cf[i + u];
-        if (packed) {
-          const P pv = ((const P*)(Vr + (long long)(i + u) * ldi))[e];
+        for (int u = 0; u < N; ++u) pv[u] = ((const P*)(Vr + (long long)(i + u) * ldi))[e];
+#pragma unroll
+        for (int u = 0; u < N; ++u)
 #pragma unroll
           for (int q = 0; q < W; ++q) {
-            const TB v = PK::get(pv, q);
-            sx[q][u] += c.x * v.x - c.y * v.y;
-            sy[q][u] += c.x * v.y + c.y * v.x;
+            const typename Acc<TB>::V c = cf[i + u];
+            const TB v = PK::get(pv[u], q);
+            sx[q][u & 3] += c.x * v.x - c.y * v.y;
+            sy[q][u & 3] += c.x * v.y + c.y * v.x;
           }
-        } else {
-          const TB v = Vr[(long long)(i + u) * ldi + e];
-          sx[0][u] += c.x * v.x - c.y * v.y;
-          sy[0][u] += c.x * v.y + c.y * v.x;
-        }
-      }
-    }
-    for (; i < k; ++i) {
-      const typename Acc<TB>::V c = cf[i];
-      if (packed) {
-        const P pv = ((const P*)(Vr + (long long)i * ldi))[e];
-#pragma unroll
-        for (int q = 0; q < W; ++q) {
-          const TB v = PK::get(pv, q);
-          sx[q][0] += c.x * v.x - c.y * v.y;
-          sy[q][0] += c.x * v.y + c.y * v.x;
-        }
       } else {
-        const TB v = Vr[(long long)i * ldi + e];
-        sx[0][0] += c.x * v.x - c.y * v.y;
-        sy[0][0] += c.x * v.y + c.y * v.x;
+        TB v[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] = Vr[(long long)(i + u) * ldi + e];
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+          const typename Acc<TB>::V c = cf[i + u];
+          sx[0][u & 3] += c.x * v[u].x - c.y * v[u].y;
+          sy[0][u & 3] += c.x * v[u].y + c.y * v[u].x;
+        }
       }
+    };
+    int i = 0;
+    for (; i + 8 <= k; i += 8) terms(i, std::integral_constant<int, 8>{});
+    if (i + 4 <= k) {
+      terms(i, std::integral_constant<int, 4>{});
+      i += 4;
     }
+    for (; i < k; ++i) terms(i, std::integral_constant<int, 1>{});
 #pragma unroll
     for (int q = 0; q < W; ++q)
       if (q == 0 || packed) {
@@ -661,7 +711,7 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
     for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
     if (threadIdx.x == 0) {
       A.cnt[r] = 0;
-      const double us = ldexp(u, E);  // scale of the stored W_{j+1}: u / c
+      const double us = ldexp(sc[j + 1], E);  // scale of the stored W_{j+1}: s_{j+1} / c
       sc[j + 1] = us;
       const double nw2 = nonneg(us * us * t);  // |w'|^2 at true scale
       nw2s = nw2;
@@ -883,7 +933,9 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
   // their reductions finish in the last block, whatever the block count
   const long long packs = (L + 1) / 2;
   const int G = (int)std::max<long long>(1, std::min<long long>((packs + kRedThreads - 1) / kRedThreads, kRedBlocks));
-  const dim3 ewg(ew_blocks(L), nb), redg(G, nb);
+  // the inner products keep two blocks an SM resident: one wave of them, whose
+  // partial sums the last block also adds sooner
+  const dim3 ewg(ew_blocks(L), nb), redg(G, nb), dotg(std::min(G, kRedBlocks / 2), nb);
   vie_status s = ensure_mirror(P, nb);
   if (s != VIE_OK) return s;
   ArnState* mirror = (ArnState*)P->arn_host;
@@ -947,7 +999,7 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
       r0 = r1;
     }
     for (int pass = 0; pass < 2; ++pass) {
-      k_arn_dots<TB><<<redg, kRedThreads, 0, ss>>>(V, ldi, j, L, A, pass);
+      k_arn_dots<TB><<<dotg, kRedThreads, 0, ss>>>(V, ldi, j, L, A, pass);
       VIE_CK(cudaGetLastError());
       k_arn_axpy<TB><<<redg, kRedThreads, 0, ss>>>(V, ldi, j, L, A, pass);
       VIE_CK(cudaGetLastError());
