@@ -80,6 +80,7 @@ __device__ __forceinline__ void slab_async(E* slab, const E* src, int narr, int 
 template <typename T, int R1, int R2>
 __global__ void __launch_bounds__(256) f_p1(const typename IOT<T>::E* __restrict__ x, typename CT<T>::V* __restrict__ A,
                                             int n, int C, const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
   constexpr int M = F::M, L = 256 / R2;
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(256) f_p1(const typename IOT<T>::E* __restrict
 template <typename T, int R1, int R2, int S>
 __global__ void __launch_bounds__(256) f_py(const typename CT<T>::V* __restrict__ in, typename CT<T>::V* __restrict__ out,
                                             int n, int C, int ncomp, const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
   constexpr int M = F::M, L = 256 / R2;
@@ -208,6 +210,7 @@ template <typename T, int R1, int R2, int MODE, int NP>
 __global__ void __launch_bounds__(NP * R2 * (ModeDim<MODE>::CI > ModeDim<MODE>::CO ? ModeDim<MODE>::CI : ModeDim<MODE>::CO))
 f_p3b(typename CT<T>::V* __restrict__ B, int n, int C, const typename CT<T>::V* __restrict__ K,
       const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
   constexpr int CI = ModeDim<MODE>::CI, CO = ModeDim<MODE>::CO, NT = ModeDim<MODE>::NT;
@@ -329,6 +332,7 @@ template <typename T, int R1, int R2, int MODE, int NP>
 __global__ void __launch_bounds__(P3cThreads<T, R1, R2, MODE, NP>::N, P3cThreads<T, R1, R2, MODE, NP>::MINB)
 f_p3c(typename CT<T>::V* __restrict__ B, int n, int C, const typename CT<T>::V* __restrict__ K,
       const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
   constexpr int CI = ModeDim<MODE>::CI, CO = ModeDim<MODE>::CO, NT = ModeDim<MODE>::NT;
@@ -448,6 +452,7 @@ struct P3pThreads {
 template <int R1, int R2, int MODE, int NP>
 __global__ void __launch_bounds__(P3pThreads<MODE, NP, R2>::N, P3pThreads<MODE, NP, R2>::MINB)
 f_p3p(float2* __restrict__ B, int n, int C, const float2* __restrict__ K, const float2* __restrict__ twg) {
+  after_previous();
   typedef f32x2 T;
   typedef c32x2 V;
   typedef Fft2<T, R1, R2> F;
@@ -586,6 +591,7 @@ struct P3tThreads {
 template <int R1, int R2, int MODE, int NP>
 __global__ void __launch_bounds__(P3tThreads<MODE, NP, R2>::N)
 f_p3t(float2* __restrict__ B, int n, int C, const float2* __restrict__ K, const float2* __restrict__ twg) {
+  after_previous();
   typedef float T;
   typedef float2 V;
   typedef Fft2<T, R1, R2> F;
@@ -821,6 +827,7 @@ __device__ __forceinline__ float2 pcmulc(float2 a, float2 w) {
 template <int R1, int R2, int MODE, int NP, int MINB>
 __global__ void __launch_bounds__(NP * R2, MINB)
 f_p3s(float2* __restrict__ B, int n, int C, const float2* __restrict__ K, const float2* __restrict__ twg) {
+  after_previous();
   typedef float T;
   typedef float2 V;
   typedef Fft2<T, R1, R2> F;
@@ -1353,6 +1360,7 @@ __global__ void __launch_bounds__(256) f_p5(const typename CT<T>::V* __restrict_
                                             int n, int C, int cout, const typename CT<T>::V* __restrict__ He,
                                             const typename CT<T>::V* __restrict__ Hm, int with_identity,
                                             const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
   constexpr int M = F::M, L = 256 / R2, H2 = R1 / 2;
@@ -1447,8 +1455,7 @@ struct FastPath {
   typedef typename IOT<T>::E E;
   static vie_status p1(const E* x, V* A, int n, int C, int cin, int nrhs, const V* tw, cudaStream_t st) {
     VIE_CK(allow_smem(f_p1<T, R1, R2>));
-    f_p1<T, R1, R2><<<dim3((n * n + L - 1) / L, cin, nrhs), 256, smem(), st>>>(x, A, n, C, tw);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(launch_after(f_p1<T, R1, R2>, dim3((n * n + L - 1) / L, cin, nrhs), 256, smem(), st, x, A, n, C, tw));
     return VIE_OK;
   }
   template <int S>
@@ -1457,8 +1464,7 @@ struct FastPath {
       return VIE_EINVAL;  // not dispatched here
     } else {
       VIE_CK(allow_smem(f_py<T, R1, R2, S>));
-      f_py<T, R1, R2, S><<<dim3(M / L, n, nrhs * nc), 256, smem(), st>>>(in, out, n, C, nc, tw);
-      VIE_CK(cudaGetLastError());
+      VIE_CK(launch_after(f_py<T, R1, R2, S>, dim3(M / L, n, nrhs * nc), 256, smem(), st, in, out, n, C, nc, tw));
       return VIE_OK;
     }
   }
@@ -1472,8 +1478,7 @@ struct FastPath {
       return VIE_EINVAL;
     }
     VIE_CK(allow_smem(f_p3b<T, R1, R2, MODE, NP>));
-    f_p3b<T, R1, R2, MODE, NP><<<dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st>>>(B, n, C, K, tw);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(launch_after(f_p3b<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st, B, n, C, K, tw));
     return VIE_OK;
   }
   template <int MODE, int NP>
@@ -1492,8 +1497,7 @@ struct FastPath {
     } else {
       if (sm > cap || sm > smem_optin()) return VIE_OK;
       VIE_CK(allow_smem(f_p3c<T, R1, R2, MODE, NP>));
-      f_p3c<T, R1, R2, MODE, NP><<<dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st>>>(B, n, C, K, tw);
-      VIE_CK(cudaGetLastError());
+      VIE_CK(launch_after(f_p3c<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, B, n, C, K, tw));
       *done = true;
       return VIE_OK;
     }
@@ -1516,9 +1520,7 @@ struct FastPath {
       } else {
         if (sm > cap || sm > smem_optin()) return VIE_OK;
         VIE_CK(allow_smem(f_p3p<R1, R2, MODE, NP>));
-        f_p3p<R1, R2, MODE, NP><<<dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st>>>(
-            (float2*)B, n, C, (const float2*)K, (const float2*)tw);
-        VIE_CK(cudaGetLastError());
+        VIE_CK(launch_after(f_p3p<R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
       }
@@ -1553,9 +1555,7 @@ struct FastPath {
           if (per < 1) return VIE_OK;
           groups = std::min(groups, sms * per);
         }
-        f_p3t<R1, R2, MODE, NP><<<dim3(groups, nrhs), NTHR, sm, st>>>(
-            (float2*)B, n, C, (const float2*)K, (const float2*)tw);
-        VIE_CK(cudaGetLastError());
+        VIE_CK(launch_after(f_p3t<R1, R2, MODE, NP>, dim3(groups, nrhs), NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
       }
@@ -1580,8 +1580,7 @@ struct FastPath {
         // the whole unified L1 as shared memory: MINB CTAs of ~75 KB per SM
         VIE_CK(allow_smem(kern, true));
         const int groups = (M / 2 + 1) * (NTX / 2);
-        kern<<<dim3(groups, nrhs), Cfg::NTHR, sm, st>>>((float2*)B, n, C, (const float2*)K, (const float2*)tw);
-        VIE_CK(cudaGetLastError());
+        VIE_CK(launch_after(kern, dim3(groups, nrhs), Cfg::NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
       }
@@ -1693,10 +1692,10 @@ struct FastPath {
     } else {
       if (cout <= 3) {
         VIE_CK(allow_smem(f_p5<T, R1, R2, 3>));
-        f_p5<T, R1, R2, 3><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+        VIE_CK(launch_after(f_p5<T, R1, R2, 3>, grid, 256, smem(), st, A, xin, y, n, C, cout, He, Hm, wid, tw));
       } else {
         VIE_CK(allow_smem(f_p5<T, R1, R2, 6>));
-        f_p5<T, R1, R2, 6><<<grid, 256, smem(), st>>>(A, xin, y, n, C, cout, He, Hm, wid, tw);
+        VIE_CK(launch_after(f_p5<T, R1, R2, 6>, grid, 256, smem(), st, A, xin, y, n, C, cout, He, Hm, wid, tw));
       }
       VIE_CK(cudaGetLastError());
       return VIE_OK;

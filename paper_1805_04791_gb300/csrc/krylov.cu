@@ -420,6 +420,7 @@ __device__ __forceinline__ void arn_chunk(const TB* V, long long ldi, const TB* 
 template <typename TB>
 __global__ void __launch_bounds__(kRedThreads) k_arn_dots(const TB* __restrict__ V, long long ldi, int j, long long L,
                                                           ArnLayout A, int pass) {
+  after_previous();
   typedef typename Acc<TB>::T AT;
   typedef typename Pack<TB>::P P;
   constexpr int W = Pack<TB>::W;
@@ -599,13 +600,17 @@ __device__ void arn_finalize(ArnLayout& A, int r, int j, const double2* h0, cons
 // latency was most of a short vector's step).
 template <typename TB>
 __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, long long ldi, int j, long long L,
-                                                          ArnLayout A, int pass) {
+                                                          ArnLayout A, int pass, ArnState* mirror) {
+  after_previous();
   typedef typename Acc<TB>::T AT;
   __shared__ typename Acc<TB>::V cf[256];
   __shared__ double red[kRedThreads / 32];
   const int r = blockIdx.y, G = gridDim.x, m = A.m, ldp = m + 3;
   ArnState* S = A.st + r;
-  if (S->done || (pass == 1 && !S->reorth)) return;  // block-uniform
+  if (S->done || (pass == 1 && !S->reorth)) {  // block-uniform
+    if (mirror && blockIdx.x == 0 && threadIdx.x == 0) mirror[r] = *S;
+    return;
+  }
   double* sc = A.sc + (long long)r * (m + 2);
   const int k = j + 1;
   const typename Acc<TB>::V* cg = (const typename Acc<TB>::V*)(A.coef + (long long)r * m);
@@ -727,6 +732,7 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
     const double2* h0 = A.hcol + (long long)r * 2 * (m + 2);
     arn_finalize(A, r, j, h0, pass == 1 ? h0 + (m + 2) : nullptr, sqrt(nw2s));
   }
+  if (mirror && threadIdx.x == 0) mirror[r] = *S;  // thread 0 wrote the state
 }
 
 // Start of a cycle: state of member r from its residual norm beta and threshold.
@@ -984,7 +990,8 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
   };
   // One step: the apply (on contiguous runs of members not yet seen as done when
   // `compact`; members that finished within the last kArnLag steps still ride
-  // along, harmlessly), both Gram-Schmidt passes, and the state copy + event.
+  // along, harmlessly), both Gram-Schmidt passes (the second stores the state in
+  // pinned host memory), and the event that marks it complete.
   auto enqueue_step = [&](int j, cudaStream_t ss, bool compact, bool capturing) -> vie_status {
     for (int r0 = 0; r0 < nb;) {
       if (compact && !cur.empty() && cur[r0].done) {
@@ -999,13 +1006,9 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
       r0 = r1;
     }
     for (int pass = 0; pass < 2; ++pass) {
-      k_arn_dots<TB><<<dotg, kRedThreads, 0, ss>>>(V, ldi, j, L, A, pass);
-      VIE_CK(cudaGetLastError());
-      k_arn_axpy<TB><<<redg, kRedThreads, 0, ss>>>(V, ldi, j, L, A, pass);
-      VIE_CK(cudaGetLastError());
+      VIE_CK(launch_after(k_arn_dots<TB>, dotg, kRedThreads, 0, ss, V, ldi, j, L, A, pass));
+      VIE_CK(launch_after(k_arn_axpy<TB>, redg, kRedThreads, 0, ss, V, ldi, j, L, A, pass, pass == 1 ? mirror + (size_t)(j % kArnSlots) * nb : nullptr));
     }
-    VIE_CK(cudaMemcpyAsync(mirror + (size_t)(j % kArnSlots) * nb, A.st, sizeof(ArnState) * nb,
-                           cudaMemcpyDeviceToHost, ss));
     // inside a stream capture the record must be External to become an event-record
     // node of the graph (a plain one only expresses a dependency within the capture)
     if (capturing) VIE_CK(cudaEventRecordWithFlags(P->arn_ev[j % kArnSlots], ss, cudaEventRecordExternal));

@@ -15,6 +15,14 @@
 
 namespace vie {
 
+// First statement of a kernel launched by launch_after (vie_internal.h): lets the
+// next kernel of the stream be placed on the SMs as soon as every block of this
+// grid has started, then waits for the grids before this one to complete.
+// Nothing is read or written before it.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
+}
+
 // ------------------------------------------------------------ complex math
 __host__ __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }

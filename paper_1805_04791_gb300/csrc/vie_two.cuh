@@ -182,6 +182,7 @@ template <typename T, int RM>
 __global__ void __launch_bounds__(256) k2_p1(const typename IOT<T>::E* __restrict__ x, typename CT<T>::V* __restrict__ A,
                                              int n, TwoPlan p, int LS, int C,
                                              const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef typename CT<T>::V V;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* tw = (V*)smraw;
@@ -209,6 +210,7 @@ template <typename T, int RM, int S>
 __global__ void __launch_bounds__(sizeof(typename CT<T>::V) == 8 ? 384 : 192, 2) k2_py(const typename CT<T>::V* __restrict__ in, typename CT<T>::V* __restrict__ out,
                                              int n, TwoPlan p, int LS, int C, int ncomp,
                                              const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef typename CT<T>::V V;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* tw = (V*)smraw;
@@ -296,6 +298,7 @@ template <typename T, int RM, int MODE>
 __global__ void __launch_bounds__(TwoP3<T, RM, MODE>::N, TwoP3<T, RM, MODE>::MINB)
 k2_p3(typename CT<T>::V* __restrict__ B, int n, TwoPlan p, int LS, int C, int mode_rt,
       const typename CT<T>::V* __restrict__ K, const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef typename CT<T>::V V;
   const int mode = MODE < 0 ? mode_rt : MODE;
   const int CI = mode == KM_MAXWELL6 ? 6 : 3, CO = mode == KM_SYM3 ? 3 : (mode == KM_DIV ? 1 : 6);
@@ -393,6 +396,7 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(TwoP3<T, 16, MODE>::N, TwoP3<T, 16, MODE>::MINB)
 k2_p3h(typename CT<T>::V* __restrict__ B, int n, TwoPlan p, int LS, int C, int mode_rt,
        const typename CT<T>::V* __restrict__ K, const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef typename CT<T>::V V;
   const int mode = MODE < 0 ? mode_rt : MODE;
   const int CI = mode == KM_MAXWELL6 ? 6 : 3, CO = mode == KM_SYM3 ? 3 : (mode == KM_DIV ? 1 : 6);
@@ -534,6 +538,7 @@ __global__ void __launch_bounds__(256, sizeof(typename CT<T>::V) == 8 ? 2 : 1) k
                                              const typename CT<T>::V* __restrict__ He,
                                              const typename CT<T>::V* __restrict__ Hm, int with_identity,
                                              const typename CT<T>::V* __restrict__ twg) {
+  after_previous();
   typedef typename CT<T>::V V;
   typedef typename IOT<T>::E E;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -607,17 +612,16 @@ vie_status two_line_pass(int pass, const TwoPlan& p, const TwoArgs& a, cudaStrea
   if (pass == 1) {
     const int rows = std::max(1, 256 / p.R1), LS = (p.R1 * p.PF) | 1;
     VIE_CK(allow_smem(k2_p1<T, RM>));
-    k2_p1<T, RM><<<dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p, rows, LS), st>>>(
-        (const typename IOT<T>::E*)a.x, (V*)a.A, n, p, LS, a.C, tw);
+    VIE_CK(launch_after(k2_p1<T, RM>, dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p, rows, LS), st, (const typename IOT<T>::E*)a.x, (V*)a.A, n, p, LS, a.C, tw));
   } else {
     const int nl = sizeof(V) == 8 ? 16 : 8, LS = two_pitch(p, nl, sizeof(V)), nc = pass == 2 ? a.cin : a.cout;
     const dim3 grid((M + nl - 1) / nl, n, a.nrhs * nc), blk(nl, p.R1);
     if (pass == 2) {
       VIE_CK(allow_smem(k2_py<T, RM, -1>));
-      k2_py<T, RM, -1><<<grid, blk, two_smem<V>(p, nl, LS), st>>>((const V*)a.A, (V*)a.B, n, p, LS, a.C, nc, tw);
+      VIE_CK(launch_after(k2_py<T, RM, -1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.A, (V*)a.B, n, p, LS, a.C, nc, tw));
     } else {
       VIE_CK(allow_smem(k2_py<T, RM, 1>));
-      k2_py<T, RM, 1><<<grid, blk, two_smem<V>(p, nl, LS), st>>>((const V*)a.B, (V*)a.A, n, p, LS, a.C, nc, tw);
+      VIE_CK(launch_after(k2_py<T, RM, 1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.B, (V*)a.A, n, p, LS, a.C, nc, tw));
     }
   }
   VIE_CK(cudaGetLastError());
@@ -628,22 +632,23 @@ template <typename T, int RM>
 vie_status two_z_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   typedef typename CT<T>::V V;
   TwoPlan h = p;
-  // FP32 with six lines a pencil: the halves' lines leave room for one CTA an SM
-  const bool half = RM > 16 && make_two_plan(p.M / 2, &h) && h.R1 <= 16 && !(sizeof(V) == 8 && a.C == 6);
+  bool half = RM > 16 && make_two_plan(p.M / 2, &h) && h.R1 <= 16;
+  auto smem_of = [&](int nl) {
+    return sizeof(V) * (p.M + (size_t)a.C * (half ? 2 : 1) * nl * two_pitch(h, nl, sizeof(V)));
+  };
+  // FP32 with six lines a pencil: half lines only while two CTAs share an SM (100^3
+  // with mu 299 us against 383, 150^3 1640 against 1080)
+  if (half && sizeof(V) == 8 && a.C == 6 && smem_of(TwoP3<T, RM, KM_SYM3>::NL) > 112 * 1024) half = false;
   if (!half) h = p;
   if (std::is_same<T, df>::value && RM > 16 && !half) return VIE_EINVAL;  // see two_z_fits
-  const size_t lines = (size_t)a.C * (half ? 2 : 1);
-  auto smem_of = [&](int nl) { return sizeof(V) * (p.M + lines * nl * two_pitch(h, nl, sizeof(V))); };
   int nl = TwoP3<T, RM, KM_SYM3>::NL;
   const int tz = std::is_same<T, df>::value ? a.C : 3;
   while (nl > 1 && smem_of(nl) > (size_t)smem_optin_bytes()) nl >>= 1;
-  if (sizeof(V) == 8 && nl > 4 && smem_of(nl) > 112 * 1024) nl = 4;  // two CTAs an SM
   const int LS = two_pitch(h, nl, sizeof(V));
   const dim3 grid(2 * ((p.M + nl - 1) / nl) * (p.M / 2 + 1), a.nrhs), blk(nl, h.R1, tz);
   auto go = [&](auto kern) -> vie_status {
     VIE_CK(allow_smem(kern));
-    kern<<<grid, blk, smem_of(nl), st>>>((V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K, (const V*)a.tw);
-    VIE_CK(cudaGetLastError());
+    VIE_CK(launch_after(kern, grid, blk, smem_of(nl), st, (V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K, (const V*)a.tw));
     return VIE_OK;
   };
   if constexpr (std::is_same<T, df>::value) {  // the operator's kernel sets only
@@ -653,8 +658,8 @@ vie_status two_z_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
     constexpr bool f64 = std::is_same<T, double>::value;  // the scattered field's sets are FP64 only
     if constexpr (RM > 16) {
       if (half && a.mode == KM_SYM3) return go(k2_p3h<T, KM_SYM3>);
+      if (half && a.mode == KM_MAXWELL6) return go(k2_p3h<T, KM_MAXWELL6>);
       if constexpr (f64) {
-        if (half && a.mode == KM_MAXWELL6) return go(k2_p3h<T, KM_MAXWELL6>);
         if (half && a.mode == KM_DIV) return go(k2_p3h<T, KM_DIV>);
         if (half) return go(k2_p3h<T, KM_EMRED>);
       }
@@ -674,11 +679,7 @@ vie_status two_last_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   int rows = std::max(1, 256 / (p.R1 * tz));
   while (rows > 1 && two_smem<V>(p, (size_t)a.cout * rows, LS) > 100 * 1024) --rows;
   VIE_CK(allow_smem(k2_p5<T, RM>));
-  k2_p5<T, RM><<<dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz),
-                 two_smem<V>(p, (size_t)a.cout * rows, LS), st>>>(
-      (const V*)a.A, (const E*)a.x, (E*)a.y, a.n, p, LS, a.C, a.cout, (const V*)a.He, (const V*)a.Hm, a.with_identity,
-      (const V*)a.tw);
-  VIE_CK(cudaGetLastError());
+  VIE_CK(launch_after(k2_p5<T, RM>, dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz), two_smem<V>(p, (size_t)a.cout * rows, LS), st, (const V*)a.A, (const E*)a.x, (E*)a.y, a.n, p, LS, a.C, a.cout, (const V*)a.He, (const V*)a.Hm, a.with_identity, (const V*)a.tw));
   return VIE_OK;
 }
 
