@@ -70,6 +70,20 @@ __device__ __forceinline__ void slab_async(E* slab, const E* src, int narr, int 
   cp_async_commit();
 }
 
+// Bring the rows of a pencil tile (one run of at most 8 pencils, 64 bytes, per z and
+// component) towards L2.  The half-spectrum z pass at 2n = 512 loads a component
+// at a time between its transforms, with eight warps an SM to wait for HBM:
+// prefetching the next tile takes it from 6.95 to 6.78 ms at Maxwell 256^3 with mu.
+// The z passes with more warps and smaller grids (f_p3s, f_p3c, f_p3t) gain nothing
+// or lose up to 3 %.
+__device__ __forceinline__ void prefetch_tile(const float2* base, int ncomp, int nz, long long cs, long long zs, int tid,
+                                              int nthr) {
+  for (int r = tid; r < ncomp * nz; r += nthr) {
+    const int c = r / nz, z = r - c * nz;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(base + c * cs + z * zs));
+  }
+}
+
 // ------------------------------------------------ register-resident fast path
 // For 2n = R1 * R2 in {64, 96, 128, 192, 256, 384, 512} every line is transformed by R2
 // threads with one shared-memory transpose per direction (vie_fft2.cuh).
@@ -1173,6 +1187,12 @@ f_p3h(float2* __restrict__ B, int C, const float2* __restrict__ K, const float2*
     const int ky = (v & 1) ? M - kyp : kyp;
     const int kx = ((v & 2) ? NTX - 1 - txp : txp) * NP + l;
     V* colbase = tile_base(grp, v);
+    {
+      const int vp = self_y ? (v == 0 ? 2 : 4) : v + 1;
+      if (vp < 4)
+        prefetch_tile(tile_base(grp, vp) - l - (long long)(h * G) * cs + (long long)r * (NN / 2) * zs, NG * G, NN / 2, cs, zs,
+                      threadIdx.x, NTHR);
+    }
     __syncthreads();  // twiddle table written; the previous tile's readers of the lines are done
     // ---- forward: step 1 of every component into its line, step 2 from the lines
 #pragma unroll
