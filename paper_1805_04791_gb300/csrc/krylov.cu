@@ -105,6 +105,7 @@ static const int kRedThreads = 256;
 __host__ __device__ static inline double nonneg(double v) { return v < 0.0 ? 0.0 : v; }
 
 static const int kDotChunk = 8;
+static const int kGroupMax = 64;  // right-hand sides of a lockstep group
 static const int kArnSlots = 8;  // pinned state copies in flight (steps)
 static const int kArnLag = 2;    // steps the host may issue past the state it has read
 static_assert(kArnSlots == (int)(sizeof(((vie_problem*)nullptr)->arn_ev) / sizeof(cudaEvent_t)), "event slots");
@@ -907,15 +908,9 @@ static bool arnoldi_shift() {
 }
 
 // Pinned host mirror of the group's per-member state, one slot per step in flight.
-static vie_status ensure_mirror(vie_problem* P, int nb) {
-  const size_t need = sizeof(ArnState) * (size_t)nb * kArnSlots;
-  if (P->arn_host_bytes < need) {
-    if (P->arn_host) cudaFreeHost(P->arn_host);
-    P->arn_host = nullptr;
-    P->arn_host_bytes = 0;
-    VIE_CK(cudaMallocHost(&P->arn_host, need));
-    P->arn_host_bytes = need;
-  }
+static vie_status ensure_mirror(vie_problem* P) {
+  static_assert(sizeof(ArnState) * kGroupMax * kArnSlots <= kPinnedBytes, "mirror fits a pinned block");
+  if (!P->arn_host) VIE_CK(pinned_take(&P->arn_host));
   for (int i = 0; i < kArnSlots; ++i)
     if (!P->arn_ev[i]) VIE_CK(cudaEventCreateWithFlags(&P->arn_ev[i], cudaEventDisableTiming));
   return VIE_OK;
@@ -942,7 +937,7 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
   // the inner products keep two blocks an SM resident: one wave of them, whose
   // partial sums the last block also adds sooner
   const dim3 ewg(ew_blocks(L), nb), redg(G, nb), dotg(std::min(G, kRedBlocks / 2), nb);
-  vie_status s = ensure_mirror(P, nb);
+  vie_status s = ensure_mirror(P);
   if (s != VIE_OK) return s;
   ArnState* mirror = (ArnState*)P->arn_host;
   ArnLayout A = g.A;
@@ -1171,14 +1166,14 @@ static int pick_group(vie_problem* P, int nrhs, int m, bool mixed) {
   const long long L = (long long)P->ncomp * P->n * P->n * P->n;
   size_t freeb = 0, totb = 0;
   if (cudaMemGetInfo(&freeb, &totb) != cudaSuccess) return 1;
-  freeb += P->ks.bytes + P->ws.bytes;  // our own workspaces are reusable
+  freeb += P->ks.bytes + P->ws.bytes + pool_unused();  // our own workspaces and unused memory are reusable
   const size_t per = group_bytes_per_rhs(L, m, mixed) +
                      apply_workspace_bytes(P->n, P->nk, std::max(cin_of(P->kapply.mode), cout_of(P->kapply.mode)), 1,
                                            VIE_FP64);
   long long nb = (long long)(0.8 * (double)freeb / (double)per);
   const char* cap = getenv("VIE_GROUP_MAX");
   if (cap) nb = std::min<long long>(nb, atoi(cap));
-  return (int)std::max<long long>(1, std::min<long long>(nb, std::min(nrhs, 64)));
+  return (int)std::max<long long>(1, std::min<long long>(nb, std::min(nrhs, kGroupMax)));
 }
 
 // ------------------------------------------------------------ Bi-CGStab

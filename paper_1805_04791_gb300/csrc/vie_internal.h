@@ -100,7 +100,6 @@ struct vie_problem {
   // device-resident GMRES: pinned host copies of the per-member Arnoldi state
   // (one slot per step in flight) and the events that mark each copy complete
   void* arn_host = nullptr;
-  size_t arn_host_bytes = 0;
   cudaEvent_t arn_ev[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   // single right-hand-side GMRES steps replayed as CUDA graphs (one per step
   // index), valid while every pointer and size baked into them is unchanged
@@ -118,6 +117,12 @@ void set_error(const std::string& msg);
 // concurrent problems on other streams keep running).
 cudaError_t dalloc(void** p, size_t bytes, cudaStream_t st);
 void dfree(void* p, cudaStream_t st);
+// Bytes the library's pool on the current device holds without using them.
+size_t pool_unused();
+// Pinned host block of kPinnedBytes: one from the kept ones, or a new one; and back.
+static const size_t kPinnedBytes = 64 * 1024;
+cudaError_t pinned_take(void** p);
+void pinned_give(void* p);
 vie_status cuda_fail(cudaError_t e, const char* what);
 // Whether the byte ranges [a, a + na) and [b, b + nb) share a byte.
 bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb);
