@@ -125,69 +125,48 @@ template <typename TB> struct Acc;
 template <> struct Acc<double2> { typedef double T; typedef double2 V; };
 template <> struct Acc<float2> { typedef float T; typedef float2 V; };
 
-// partial[(r * ldp + i) * G + block] = block's share of conj(V_i[r]) w[r], i < k;
-// with_self: slot k gets conj(w[r]) w[r].  grid = (G, nb).
-template <typename TB>
-__global__ void __launch_bounds__(kRedThreads) k_multidot(const TB* __restrict__ V, long long ldi, int k,
-                                                          const TB* __restrict__ w, long long L, double2* partial,
-                                                          int ldp, int with_self) {
-  typedef typename Acc<TB>::T AT;
-  __shared__ double2 red[kRedThreads / 32][kDotChunk];
-  const int G = gridDim.x, r = blockIdx.y;
-  const TB* Vr = V + (long long)r * L;
-  const TB* wr = w + (long long)r * L;
-  const int ktot = k + (with_self ? 1 : 0);
-  for (int i0 = 0; i0 < ktot; i0 += kDotChunk) {
-    const int cnt = min(kDotChunk, ktot - i0);
-    AT ar[kDotChunk], ai[kDotChunk];
+// K block sums in FP64, one warp a value: every thread's value goes through shared
+// memory, a lane of the warp adds eight and the warp shuffles once.  A shuffle tree
+// in every warp takes four times the FP64 instructions, at 16 cycles each.  Value t
+// goes to partial[t * stride].
+template <int K>
+__device__ __forceinline__ void block_sums(const double* re, const double* im, double2* partial, long long stride) {
+  __shared__ double2 all[K][kRedThreads];
 #pragma unroll
-    for (int t = 0; t < kDotChunk; ++t) ar[t] = ai[t] = (AT)0;
-    const long long stride = (long long)G * blockDim.x;
-    long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    // two elements per iteration: twice the loads in flight per thread
-    for (; e + stride < L; e += 2 * stride) {
-      const TB wa = wr[e], wb = wr[e + stride];
+  for (int t = 0; t < K; ++t) all[t][threadIdx.x] = make_double2(re[t], im[t]);
+  __syncthreads();
+  const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (t >= K) return;
+  double2 s = all[t][lane];
 #pragma unroll
-      for (int t = 0; t < kDotChunk; ++t)
-        if (t < cnt) {
-          const int i = i0 + t;
-          const TB va = (i < k) ? Vr[(long long)i * ldi + e] : wa;
-          const TB vb = (i < k) ? Vr[(long long)i * ldi + e + stride] : wb;
-          ar[t] += va.x * wa.x + va.y * wa.y + vb.x * wb.x + vb.y * wb.y;
-          ai[t] += va.x * wa.y - va.y * wa.x + vb.x * wb.y - vb.y * wb.x;
-        }
-    }
-    for (; e < L; e += stride) {
-      const TB we = wr[e];
-#pragma unroll
-      for (int t = 0; t < kDotChunk; ++t)
-        if (t < cnt) {
-          const int i = i0 + t;
-          const TB v = (i < k) ? Vr[(long long)i * ldi + e] : we;
-          ar[t] += v.x * we.x + v.y * we.y;
-          ai[t] += v.x * we.y - v.y * we.x;
-        }
-    }
-    // warp sums in the accumulation type, for the slots in use only (cnt is
-    // block-uniform); the cross-warp and cross-block sums are FP64
-#pragma unroll
-    for (int t = 0; t < kDotChunk; ++t)
-      if (t < cnt) {
-        AT ax = ar[t], ay = ai[t];
-        for (int off = 16; off > 0; off >>= 1) {
-          ax += __shfl_down_sync(0xffffffffu, ax, off);
-          ay += __shfl_down_sync(0xffffffffu, ay, off);
-        }
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][t] = make_double2((double)ax, (double)ay);
-      }
-    __syncthreads();
-    if (threadIdx.x < cnt) {
-      double2 sm = make_double2(0, 0);
-      for (int wgi = 0; wgi < kRedThreads / 32; ++wgi) sm = sm + red[wgi][threadIdx.x];
-      partial[((long long)r * ldp + i0 + threadIdx.x) * G + blockIdx.x] = sm;
-    }
-    __syncthreads();
+  for (int q = 1; q < kRedThreads / 32; ++q) s = s + all[t][lane + 32 * q];
+  for (int off = 16; off > 0; off >>= 1) {
+    s.x += __shfl_down_sync(0xffffffffu, s.x, off);
+    s.y += __shfl_down_sync(0xffffffffu, s.y, off);
   }
+  if (lane == 0) partial[(long long)t * stride] = s;
+}
+
+// partial[(r * ldp) * G + block] = block's share of |w[r]|^2, four elements' loads in
+// flight.  grid = (G, nb).
+__global__ void __launch_bounds__(kRedThreads) k_norms(const double2* __restrict__ w, long long L, double2* partial,
+                                                       int ldp) {
+  const int G = gridDim.x, r = blockIdx.y;
+  const double2* wr = w + (long long)r * L;
+  const long long stride = (long long)G * blockDim.x;
+  double s = 0;
+  const double zero = 0;
+  long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  constexpr int U = 4;
+  for (; e + (U - 1) * stride < L; e += U * stride) {
+    double2 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) x[u] = wr[e + u * stride];
+#pragma unroll
+    for (int u = 0; u < U; ++u) s += x[u].x * x[u].x + x[u].y * x[u].y;
+  }
+  for (; e < L; e += stride) s += wr[e].x * wr[e].x + wr[e].y * wr[e].y;
+  block_sums<1>(&s, &zero, partial + (long long)r * ldp * G + blockIdx.x, G);
 }
 
 // out[r * ldo + i] = sum_b partial[(r * ldp + i) * G + b], grid = (k, nb).
@@ -856,7 +835,7 @@ static int ldp_of(const Group& g) { return g.m + 3; }
 // norms of nb vectors [r][L] (FP64) -> host
 static vie_status norms_host(const double2* v, Group& g, std::vector<double>& out, cudaStream_t st) {
   const int G = red_blocks(g.L);
-  k_multidot<double2><<<dim3(G, g.nb), kRedThreads, 0, st>>>(v, 0, 0, v, g.L, g.partial, ldp_of(g), 1);
+  k_norms<<<dim3(G, g.nb), kRedThreads, 0, st>>>(v, g.L, g.partial, ldp_of(g));
   VIE_CK(cudaGetLastError());
   k_reduce_partials<<<dim3(1, g.nb), 256, 0, st>>>(g.partial, 1, G, ldp_of(g), g.hdev, g.HS);
   VIE_CK(cudaGetLastError());
@@ -872,8 +851,8 @@ static vie_status norms_host(const double2* v, Group& g, std::vector<double>& ou
 static vie_status norms2_host(const double2* v, const double2* w, Group& g, std::vector<double>& ov,
                               std::vector<double>& ow, cudaStream_t st) {
   const int G = red_blocks(g.L);
-  k_multidot<double2><<<dim3(G, g.nb), kRedThreads, 0, st>>>(v, 0, 0, v, g.L, g.partial, ldp_of(g), 1);
-  k_multidot<double2><<<dim3(G, g.nb), kRedThreads, 0, st>>>(w, 0, 0, w, g.L, g.partial + G, ldp_of(g), 1);
+  k_norms<<<dim3(G, g.nb), kRedThreads, 0, st>>>(v, g.L, g.partial, ldp_of(g));
+  k_norms<<<dim3(G, g.nb), kRedThreads, 0, st>>>(w, g.L, g.partial + G, ldp_of(g));
   VIE_CK(cudaGetLastError());
   k_reduce_partials<<<dim3(1, g.nb), 256, 0, st>>>(g.partial, 1, G, ldp_of(g), g.hdev, g.HS);
   k_reduce_partials<<<dim3(1, g.nb), 256, 0, st>>>(g.partial + G, 1, G, ldp_of(g), g.hdev + 1, g.HS);
@@ -1179,58 +1158,79 @@ static int pick_group(vie_problem* P, int nrhs, int m, bool mixed) {
 // ------------------------------------------------------------ Bi-CGStab
 // Unpreconditioned Bi-CGStab (van der Vorst 1992), the solver the paper's
 // experiments use (Sec. 5), on the FP64 apply; two operator applies per
-// iteration.  Reductions: up to four inner products conj(a_i) b_i per pass.
+// iteration.  Reductions: one or two inner products conj(a_i) b_i per pass.
 struct Dots4 {
   const double2* a[4];
   const double2* b[4];
   int k;
 };
 
+// Block partials of K inner products conj(a_t) b_t, four elements' loads in flight;
+// a product of a vector with itself takes its real part only.  Bi-CGStab at 70^3 (L =
+// 1.03 M): 62 -> 26 us a launch on average.
+template <int K>
 __global__ void __launch_bounds__(kRedThreads) k_dots4(Dots4 d, long long L, double2* partial) {
-  __shared__ double2 red[kRedThreads / 32][4];
-  double ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0};
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < L; e += (long long)gridDim.x * blockDim.x)
+  double ar[K], ai[K];
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
-      if (t < d.k) {
-        const double2 x = d.a[t][e], y = d.b[t][e];
-        ar[t] += x.x * y.x + x.y * y.y;
-        ai[t] += x.x * y.y - x.y * y.x;
+  for (int t = 0; t < K; ++t) ar[t] = ai[t] = 0;
+  auto add = [&](int t, double2 x, double2 y) {
+    ar[t] += x.x * y.x + x.y * y.y;
+    if (d.a[t] != d.b[t]) ai[t] += x.x * y.y - x.y * y.x;  // uniform
+  };
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  constexpr int U = 4;
+  for (; e + (U - 1) * stride < L; e += U * stride) {
+    double2 x[K][U], y[K][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int t = 0; t < K; ++t) {
+        x[t][u] = d.a[t][e + u * stride];
+        y[t][u] = d.b[t][e + u * stride];
       }
 #pragma unroll
-  for (int t = 0; t < 4; ++t)
-    if (t < d.k) {  // block-uniform
-      double2 a = make_double2(ar[t], ai[t]);
-      for (int off = 16; off > 0; off >>= 1) {
-        a.x += __shfl_down_sync(0xffffffffu, a.x, off);
-        a.y += __shfl_down_sync(0xffffffffu, a.y, off);
-      }
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][t] = a;
-    }
-  __syncthreads();
-  if (threadIdx.x < d.k) {
-    double2 sm = make_double2(0, 0);
-    for (int w = 0; w < kRedThreads / 32; ++w) sm = sm + red[w][threadIdx.x];
-    partial[(long long)threadIdx.x * gridDim.x + blockIdx.x] = sm;
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int t = 0; t < K; ++t) add(t, x[t][u], y[t][u]);
   }
+  for (; e < L; e += stride)
+#pragma unroll
+    for (int t = 0; t < K; ++t) add(t, d.a[t][e], d.b[t][e]);
+  block_sums<K>(ar, ai, partial + blockIdx.x, gridDim.x);
 }
 
-// y = a0 x0 + a1 x1 + a2 x2 (x_i may be null; y may alias x0)
-__global__ void k_lincomb(double2* y, const double2* x0, double2 a0, const double2* x1, double2 a1, const double2* x2,
-                          double2 a2, long long L) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < L; e += (long long)gridDim.x * blockDim.x) {
-    double2 v = make_double2(0, 0);
-    if (x0) v = v + cmul(a0, x0[e]);
-    if (x1) v = v + cmul(a1, x1[e]);
-    if (x2) v = v + cmul(a2, x2[e]);
-    y[e] = v;
+// y = a0 x0 + a1 x1 (+ a2 x2 if N = 3; y may alias x0), four elements' loads in flight.
+template <int N>
+__global__ void __launch_bounds__(256) k_lincomb(double2* y, const double2* x0, double2 a0, const double2* x1, double2 a1,
+                                                 const double2* x2, double2 a2, long long L) {
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  auto one = [&](double2 p0, double2 p1, double2 p2) {
+    const double2 v = cmul(a0, p0) + cmul(a1, p1);
+    return N == 3 ? v + cmul(a2, p2) : v;
+  };
+  const double2 zero = make_double2(0, 0);
+  constexpr int U = 4;
+  for (; e + (U - 1) * stride < L; e += U * stride) {
+    double2 p[3][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      p[0][u] = x0[e + u * stride];
+      p[1][u] = x1[e + u * stride];
+      p[2][u] = N == 3 ? x2[e + u * stride] : zero;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) y[e + u * stride] = one(p[0][u], p[1][u], p[2][u]);
   }
+  for (; e < L; e += stride) y[e] = one(x0[e], x1[e], N == 3 ? x2[e] : zero);
 }
 
 static vie_status dots_host(Dots4 d, long long L, double2* partial, double2* dev, std::vector<cd>& out,
                             cudaStream_t st) {
   const int G = red_blocks(L);
-  k_dots4<<<G, kRedThreads, 0, st>>>(d, L, partial);
+  if (d.k == 1) k_dots4<1><<<G, kRedThreads, 0, st>>>(d, L, partial);
+  else k_dots4<2><<<G, kRedThreads, 0, st>>>(d, L, partial);
   VIE_CK(cudaGetLastError());
   k_reduce_partials<<<dim3(d.k, 1), 256, 0, st>>>(partial, d.k, G, 0, dev, 0);
   VIE_CK(cudaGetLastError());
@@ -1312,7 +1312,7 @@ static vie_status run_bicgstab(vie_problem* P, const void* rhs, void* Jv, const 
       const cd beta = (rho_new / rho) * (alpha / omega);
       rho = rho_new;
       // p = r + beta (p - omega v)
-      k_lincomb<<<eb, 256, 0, st>>>(p, r, one, p, C(beta), v, C(-beta * omega), L);
+      k_lincomb<3><<<eb, 256, 0, st>>>(p, r, one, p, C(beta), v, C(-beta * omega), L);
       s = run_apply(P, P->kapply, p, v, VIE_FP64, 1, true, st);
       if (s != VIE_OK) return s;
       ++inf->applies_fp64;
@@ -1320,12 +1320,12 @@ static vie_status run_bicgstab(vie_problem* P, const void* rhs, void* Jv, const 
       s = dots_host(q, L, partial, dev, d, st);
       if (s != VIE_OK) return s;
       alpha = rho / d[0];
-      k_lincomb<<<eb, 256, 0, st>>>(sv, r, one, v, C(-alpha), nullptr, zero, L);
+      k_lincomb<2><<<eb, 256, 0, st>>>(sv, r, one, v, C(-alpha), nullptr, zero, L);
       q = Dots4{{sv, nullptr, nullptr, nullptr}, {sv, nullptr, nullptr, nullptr}, 1};
       s = dots_host(q, L, partial, dev, d, st);
       if (s != VIE_OK) return s;
       if (std::sqrt(nonneg(d[0].real())) / nb <= opt->tol) {
-        k_lincomb<<<eb, 256, 0, st>>>(x, x, one, p, C(alpha), nullptr, zero, L);
+        k_lincomb<2><<<eb, 256, 0, st>>>(x, x, one, p, C(alpha), nullptr, zero, L);
         rel = std::sqrt(nonneg(d[0].real())) / nb;
         conv = true;
         ++inf->inner_iters;
@@ -1338,8 +1338,8 @@ static vie_status run_bicgstab(vie_problem* P, const void* rhs, void* Jv, const 
       s = dots_host(q, L, partial, dev, d, st);
       if (s != VIE_OK) return s;
       omega = d[0] / d[1];
-      k_lincomb<<<eb, 256, 0, st>>>(x, x, one, p, C(alpha), sv, C(omega), L);
-      k_lincomb<<<eb, 256, 0, st>>>(r, sv, one, tv, C(-omega), nullptr, zero, L);
+      k_lincomb<3><<<eb, 256, 0, st>>>(x, x, one, p, C(alpha), sv, C(omega), L);
+      k_lincomb<2><<<eb, 256, 0, st>>>(r, sv, one, tv, C(-omega), nullptr, zero, L);
       VIE_CK(cudaGetLastError());
       ++inf->inner_iters;
     }
@@ -1365,9 +1365,9 @@ static vie_status fp64_residual(vie_problem* P, const double2* b, const double2*
   double2 h[2] = {make_double2(0, 0), make_double2(0, 0)};
   if (s == VIE_OK) {
     k_bminus<<<ew_blocks(L), 256, 0, st>>>(r, b, L);
-    k_multidot<double2><<<dim3(G, 1), kRedThreads, 0, st>>>(r, 0, 0, r, L, partial, 2, 1);
+    k_norms<<<dim3(G, 1), kRedThreads, 0, st>>>(r, L, partial, 2);
     k_reduce_partials<<<dim3(1, 1), 256, 0, st>>>(partial, 1, G, 2, out, 2);
-    k_multidot<double2><<<dim3(G, 1), kRedThreads, 0, st>>>(b, 0, 0, b, L, partial, 2, 1);
+    k_norms<<<dim3(G, 1), kRedThreads, 0, st>>>(b, L, partial, 2);
     k_reduce_partials<<<dim3(1, 1), 256, 0, st>>>(partial, 1, G, 2, out + 1, 2);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, st);
