@@ -153,8 +153,8 @@ typedef struct {
  *          padded length Q >= 2 (3n) - 1 made of the factors 2, 3, 5, 7, 11.
  *          Odd n is valid: the set-up grid 3n is then odd and its frequency
  *          cut-off is the symmetric |m| <= (3n-1)/2, with no Nyquist entry.
- *          The set-up holds octant transform buffers of about 3.75 n^3 FP64
- *          complex values (8 GB at n = 512); a failed allocation returns VIE_ENOMEM.  M <= 1024
+ *          The set-up holds octant transform buffers of about 7.5 n^3 FP64
+ *          complex values (16 GB at n = 512); a failed allocation returns VIE_ENOMEM.  M <= 1024
  *          for every valid n, so the generic z-pass tile (six lines of M + 1
  *          elements at 16 bytes, FP64) fits in shared memory.
  *   lo, hi box [lo, hi]^3 (hi > lo).

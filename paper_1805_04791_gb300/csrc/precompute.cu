@@ -12,6 +12,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <cmath>
+#include <functional>
 #include <vector>
 
 #include "vie_internal.h"
@@ -224,7 +225,9 @@ __global__ void k_ghat_table(double2* tab, int jmax, double dk, double w, double
 // exchanging axes (G^ is radial): 1, -k_z^2, -k_x k_y and i k_z, z being the
 // axis that is not like the other two.
 // Measured, 192^3 reduced Maxwell problem: 302 ms for seven symbols on whole cubes
-// (279 ms of cube transforms, 21 ms to fill them), 29.5 ms for three bases here.
+// (279 ms of cube transforms, 21 ms to fill them); three bases here take 10.3 ms
+// (29.5 with the double-word sums and products of twice the instructions, 12.3
+// without the pairing in k_axis; Helmholtz 64^3 0.43 -> 0.32 ms by it).
 enum Base { BASE_1 = 0, BASE_ZZ, BASE_XY, BASE_DZ, BASE_COUNT };
 
 static int base_of(int sym) {
@@ -247,6 +250,7 @@ static int axis_of(int sym) {
 struct AxisPass {
   int axis;        // 0 x, 1 y, 2 z
   int base;        // Base
+  int pair;        // a second base, odd in this axis, in the same transforms (-1: none)
   int n, nk, sn;
   int odd;         // the base is odd in this axis
   int nl;          // lines per tile
@@ -270,14 +274,19 @@ __device__ __forceinline__ double2 base_sample(const double2* __restrict__ tab, 
   return make_double2(-oz * G.y, oz * G.x);
 }
 
+// A base that is even in the axis and one that is odd go through one transform of
+// their sum: the even part of the result is the first's, the odd part the second's
+// (-k_z^2 and -k_x k_y, of the same magnitude, in the x and y passes).
+//
 // One line operator over `nl` lines per CTA (blockDim.y = nl, blockDim.x threads
 // a line).  Layouts: x pass  tab -> out [mz][my][kx], y pass [mz][my][kx] ->
 // [mz][ky][kx], z pass [mz][ky][kx] -> [kz][ky][kx]; 0 <= m <= sn/2, 0 <= k <= nk.
 // The lines of a y or z tile are neighbours in kx, so a tile reads and writes
 // runs of nl 16-byte values.
 template <typename T>
-__global__ void k_axis(const double2* __restrict__ in, double2* __restrict__ out, AxisPass q,
-                       const typename CT<T>::V* __restrict__ tws, const typename CT<T>::V* __restrict__ twm) {
+__global__ void k_axis(const double2* __restrict__ in, double2* __restrict__ out, const double2* __restrict__ in2,
+                       double2* __restrict__ out2, AxisPass q, const typename CT<T>::V* __restrict__ tws,
+                       const typename CT<T>::V* __restrict__ twm) {
   typedef typename CT<T>::V V;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nl = q.nl, LS = q.LS, sn = q.sn, n = q.n, M = q.pm.M, Q = q.ps.Q, O = q.nk + 1, S = sn / 2 + 1;
@@ -300,18 +309,25 @@ __global__ void k_axis(const double2* __restrict__ in, double2* __restrict__ out
     int l, m;
     if (q.axis == 0) { l = idx / S; m = idx - l * S; } else { m = idx / nl; l = idx - m * nl; }
     const long long r = r0 + l;
-    double2 v = make_double2(0.0, 0.0);
+    double2 v = make_double2(0.0, 0.0), v2 = v;
     if (r < lines) {
       if (q.axis == 0) {
         const int mz = (int)(r / S), my = (int)(r - (long long)mz * S);
         v = base_sample(in, q.base, m, my, mz, sn, q.dk);
+        if (q.pair >= 0) v2 = base_sample(in, q.pair, m, my, mz, sn, q.dk);
       } else {
         v = in[ibase + m * istep + r];
+        if (q.pair >= 0) v2 = in2[ibase + m * istep + r];
       }
     }
-    const V a = to_v<T>(v);
+    V a = to_v<T>(v), am = q.odd ? vneg(a) : a;  // at m and at -m
+    if (q.pair >= 0) {
+      const V c = to_v<T>(v2);
+      am = a - c;
+      a = a + c;
+    }
     b0[l * LS + m] = a;
-    if (m > 0 && 2 * m != sn) b0[l * LS + sn - m] = q.odd ? vneg(a) : a;
+    if (m > 0 && 2 * m != sn) b0[l * LS + sn - m] = am;
   }
   __syncthreads();
   V* r = line_fft<+1, T>(b0, b1, q.ps, ts, tws + Q, nl, LS);
@@ -328,19 +344,26 @@ __global__ void k_axis(const double2* __restrict__ in, double2* __restrict__ out
     if (q.axis == 0) { l = idx / O; k = idx - l * O; } else { k = idx / nl; l = idx - k * nl; }
     const long long row = r0 + l;
     if (row >= lines) continue;
-    const double2 v = from_v<T>(w[l * LS + k]);
-    out[q.axis == 0 ? row * O + k : obase + k * ostep + row] = q.scale * v;
+    const long long at = q.axis == 0 ? row * O + k : obase + k * ostep + row;
+    const V v = w[l * LS + k];
+    if (q.pair < 0) {
+      out[at] = q.scale * from_v<T>(v);
+    } else {
+      const V vm = w[l * LS + (k == 0 ? 0 : M - k)];
+      out[at] = 0.5 * q.scale * from_v<T>(v + vm);
+      out2[at] = 0.5 * q.scale * from_v<T>(v - vm);
+    }
   }
 }
 
-// Octant of a base symbol: the three line operators.  A1 holds [S][S][O], A2 [S][O][O].
+// Octants of the bases in `mask`: the three line operators of each.  A1 holds
+// [2][S][S][O], A2 [2][S][O][O], oct [BASE_COUNT][O][O][O].
 template <typename T>
-static vie_status base_octant(vie_problem* P, int base, const double2* tab, double2* A1, double2* A2, double2* oct,
-                              const FftPlan& ps, const typename CT<T>::V* tws, const typename CT<T>::V* twm,
-                              cudaStream_t st) {
+static vie_status base_octants(vie_problem* P, unsigned mask, const double2* tab, double2* A1, double2* A2, double2* oct,
+                               const FftPlan& ps, const typename CT<T>::V* tws, const typename CT<T>::V* twm,
+                               cudaStream_t st) {
   typedef typename CT<T>::V V;
   AxisPass q;
-  q.base = base;
   q.n = P->n;
   q.nk = P->nk;
   q.sn = 3 * P->n;
@@ -365,16 +388,31 @@ static vie_status base_octant(vie_problem* P, int base, const double2* tab, doub
   int tx = 8;
   while (tx * 8 < ps.Q && 2 * tx * q.nl <= 256) tx <<= 1;
   const dim3 blk(tx, q.nl);
-  for (int axis = 0; axis < 3; ++axis) {
+  auto pass = [&](int axis, int base, int pair, const double2* src, double2* dst, const double2* src2,
+                  double2* dst2) -> vie_status {
     q.axis = axis;
+    q.base = base;
+    q.pair = pair;
     q.odd = (base == BASE_XY && axis != 2) || (base == BASE_DZ && axis == 2);
     q.scale = axis == 2 ? 1.0 / ((double)q.sn * q.sn * q.sn) : 1.0;
-    const double2* src = axis == 0 ? tab : (axis == 1 ? A1 : A2);
-    double2* dst = axis == 0 ? A1 : (axis == 1 ? A2 : oct);
     const dim3 grid = axis == 0 ? dim3((unsigned)(((long long)S * S + q.nl - 1) / q.nl))
                                 : dim3((O + q.nl - 1) / q.nl, axis == 1 ? S : O);
-    k_axis<T><<<grid, blk, smem, st>>>(src, dst, q, tws, twm);
+    k_axis<T><<<grid, blk, smem, st>>>(src, dst, src2, dst2, q, tws, twm);
     VIE_CK(cudaGetLastError());
+    return VIE_OK;
+  };
+  const long long n1 = (long long)S * S * O, n2 = (long long)S * O * O, O3 = (long long)O * O * O;
+  const unsigned both = (1u << BASE_ZZ) | (1u << BASE_XY);
+  const bool paired = (mask & both) == both;
+  for (int b = 0; b < BASE_COUNT; ++b) {
+    if (!(mask & (1u << b)) || (paired && b == BASE_XY)) continue;
+    const bool two = paired && b == BASE_ZZ;
+    const int pair = two ? BASE_XY : -1;
+    vie_status s = pass(0, b, pair, tab, A1, nullptr, A1 + n1);
+    if (s == VIE_OK) s = pass(1, b, pair, A1, A2, A1 + n1, A2 + n2);
+    if (s == VIE_OK) s = pass(2, b, -1, A2, oct + b * O3, nullptr, nullptr);
+    if (s == VIE_OK && two) s = pass(2, BASE_XY, -1, A2 + n2, oct + BASE_XY * O3, nullptr, nullptr);
+    if (s != VIE_OK) return s;
   }
   return VIE_OK;
 }
@@ -473,39 +511,35 @@ static vie_status compute_symbols(vie_problem* P, unsigned syms, cudaStream_t st
   }
   double2 *tab = nullptr, *A1 = nullptr, *A2 = nullptr, *tw_sn = nullptr;
   float2* tw_sn32 = nullptr;
+  cdf *tw_sndf = nullptr, *tw_2ndf = nullptr;
+  struct Guard {  // the scratch goes back on every way out
+    std::function<void()> f;
+    ~Guard() { f(); }
+  } guard{[&] {
+    void* all[] = {A1, A2, tab, tw_sn, tw_sn32, tw_sndf, tw_2ndf};
+    for (void* q : all) dfree(q, st);
+  }};
   const long long O = P->nk + 1, S = sn / 2 + 1, O3 = O * O * O;
   if (!P->base_oct) VIE_CK(dalloc((void**)&P->base_oct, sizeof(double2) * BASE_COUNT * O3, st));
   VIE_CK(dalloc((void**)&tab, sizeof(double2) * (jmax + 1), st));
   k_ghat_table<<<(jmax + 256) / 256, 256, 0, st>>>(tab, jmax, dk, w, P->L);
   VIE_CK(cudaGetLastError());
-  VIE_CK(dalloc((void**)&A1, sizeof(double2) * S * S * O, st));
-  VIE_CK(dalloc((void**)&A2, sizeof(double2) * S * O * O, st));
+  VIE_CK(dalloc((void**)&A1, sizeof(double2) * 2 * S * S * O, st));
+  VIE_CK(dalloc((void**)&A2, sizeof(double2) * 2 * S * O * O, st));
   vie_status s = make_line_table(plsn, &tw_sn, &tw_sn32, st);
   if (s != VIE_OK) return s;
   // the transforms run in double-word arithmetic (FP64 accuracy on the FP32
   // pipes); VIE_SETUP_FP64=1 keeps them in native FP64
   const char* e64 = getenv("VIE_SETUP_FP64");
   const bool dw = !(e64 && e64[0] == '1');
-  cdf *tw_sndf = nullptr, *tw_2ndf = nullptr;
   if (dw) {
     s = to_df(tw_sn, &tw_sndf, line_table_len(plsn), st);
     if (s == VIE_OK) s = to_df(P->tw64, &tw_2ndf, line_table_len(P->planM), st);
     if (s != VIE_OK) return s;
   }
-  for (int b = 0; b < BASE_COUNT; ++b) {
-    if (!(mask & (1u << b))) continue;
-    double2* oct = P->base_oct + b * O3;
-    s = dw ? base_octant<df>(P, b, tab, A1, A2, oct, plsn, tw_sndf, tw_2ndf, st)
-           : base_octant<double>(P, b, tab, A1, A2, oct, plsn, tw_sn, P->tw64, st);
-    if (s != VIE_OK) return s;
-  }
-  dfree(A1, st);
-  dfree(A2, st);
-  dfree(tab, st);
-  dfree(tw_sn, st);
-  dfree(tw_sn32, st);
-  dfree(tw_sndf, st);
-  dfree(tw_2ndf, st);
+  s = dw ? base_octants<df>(P, mask, tab, A1, A2, P->base_oct, plsn, tw_sndf, tw_2ndf, st)
+         : base_octants<double>(P, mask, tab, A1, A2, P->base_oct, plsn, tw_sn, P->tw64, st);
+  if (s != VIE_OK) return s;
   P->base_mask |= mask;
   return VIE_OK;
 }
