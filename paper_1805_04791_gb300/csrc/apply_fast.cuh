@@ -126,6 +126,67 @@ __global__ void __launch_bounds__(256) f_p1(const typename IOT<T>::E* __restrict
       for (int k2 = 0; k2 < R2; ++k2) dst[t + R2 * j + R1 * k2] = X[j][k2];
 }
 
+// P1 and P2 in one kernel for the small grids (FP32, M <= 96): a CTA takes one (component,
+// z) plane, whose n x-lines of M values fit in shared memory (M = 64: 19 KB, M = 96:
+// 42 KB), and transforms its M y-lines from there, half of them at a time, so that
+// A is neither written nor read and one launch is saved.  n R2 threads: all of them
+// have a task in every step.  At these sizes a pass is latency: FP32 apply at 32^3
+// 27.1 -> 23.6 us, at 48^3 49.2 -> 42.5 us, with the smaller blocks of f_p5.
+template <int R1, int R2>
+__global__ void __launch_bounds__(R1 * R2 / 2 * R2) f_p12(const float2* __restrict__ x, float2* __restrict__ B, int C,
+                                                          const float2* __restrict__ twg) {
+  after_previous();
+  typedef Fft2<float, R1, R2> F;
+  constexpr int M = F::M, n = M / 2, LS = F::LS;
+  static_assert(LS > M, "a plane row fits in a transpose line");
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* tw = (float2*)smraw;
+  float2* plane = tw + M;         // [n][LS]: transpose lines, then the plane's rows
+  float2* cols = plane + n * LS;  // [n][LS]: transpose lines of half the columns
+  load_tw(tw, twg, M);
+  const int z = blockIdx.x, c = blockIdx.y, b = blockIdx.z, nc = gridDim.y;
+  {
+    const int t = threadIdx.x % R2, l = threadIdx.x / R2;
+    const float2* src = x + (((long long)b * nc + c) * n + z) * (n * n) + l * n;
+    float2* s = plane + l * LS;
+    float2 u[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) u[n1] = n1 < R1 / 2 ? src[R2 * n1 + t] : make_float2(0.f, 0.f);
+    __syncthreads();
+    F::template fwd1<true>(u, t, s, tw);
+    __syncthreads();
+    float2 X[F::J][R2];
+    F::fwd2(X, t, s);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < F::J; ++j)
+      if (F::row(t, j))
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) s[t + R2 * j + R1 * k2] = X[j][k2];
+  }
+  __syncthreads();
+  const int l = threadIdx.x % n, t = threadIdx.x / n;
+  float2* s = cols + l * LS;
+  float2* dst = B + (((long long)b * C + c) * n + z) * (M * M) + l;
+#pragma unroll 1
+  for (int h = 0; h < M; h += n) {
+    float2 u[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1)
+      u[n1] = n1 < R1 / 2 ? plane[(R2 * n1 + t) * LS + h + l] : make_float2(0.f, 0.f);
+    if (h) __syncthreads();  // the first half's readers of the column lines are done
+    F::template fwd1<true>(u, t, s, tw);
+    __syncthreads();
+    float2 X[F::J][R2];
+    F::fwd2(X, t, s);
+#pragma unroll
+    for (int j = 0; j < F::J; ++j)
+      if (F::row(t, j))
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) dst[(t + R2 * j + R1 * k2) * M + h] = X[j][k2];
+  }
+}
+
 // y-lines.  S < 0: A [bc][z][y<n][kx] -> B [bc][z][ky][kx];  S > 0: B -> A (keep y < n).
 template <typename T, int R1, int R2, int S>
 __global__ void __launch_bounds__(256) f_py(const typename CT<T>::V* __restrict__ in, typename CT<T>::V* __restrict__ out,
@@ -1374,8 +1435,10 @@ f_p3h(float2* __restrict__ B, int C, const float2* __restrict__ K, const float2*
 
 // x-lines of all components: inverse, keep x < n, epilogue y = x + H u
 // (with_identity 1), y = H u (2: the operator minus the identity) or y = u (0).  CO = 3 (one H block) or 6 ([J; M] with H_eps and H_mu, or [E; H]).
-template <typename T, int R1, int R2, int CO>
-__global__ void __launch_bounds__(256) f_p5(const typename CT<T>::V* __restrict__ A,
+// NT threads: small grids take small blocks, so that their few rows spread over the
+// SMs (32^3: 32 blocks of 256 threads, or 128 of 64).
+template <typename T, int R1, int R2, int CO, int NT>
+__global__ void __launch_bounds__(NT) f_p5(const typename CT<T>::V* __restrict__ A,
                                             const typename IOT<T>::E* __restrict__ xin, typename IOT<T>::E* __restrict__ y,
                                             int n, int C, int cout, const typename CT<T>::V* __restrict__ He,
                                             const typename CT<T>::V* __restrict__ Hm, int with_identity,
@@ -1383,7 +1446,7 @@ __global__ void __launch_bounds__(256) f_p5(const typename CT<T>::V* __restrict_
   after_previous();
   typedef Fft2<T, R1, R2> F;
   typedef typename CT<T>::V V;
-  constexpr int M = F::M, L = 256 / R2, H2 = R1 / 2;
+  constexpr int M = F::M, L = NT / R2, H2 = R1 / 2;
   extern __shared__ __align__(16) unsigned char smraw[];
   V* tw = (V*)smraw;
   V* sm = tw + M;
@@ -1706,19 +1769,31 @@ struct FastPath {
   }
   static vie_status p5(const V* A, const E* xin, E* y, int n, int C, int cout, const V* He, const V* Hm, int wid,
                        int nrhs, const V* tw, cudaStream_t st) {
-    const dim3 grid((n * n + L - 1) / L, nrhs);
     if constexpr (std::is_same<T, df>::value || (std::is_same<T, double>::value && fp64_two_last(M))) {
       return VIE_EINVAL;  // not dispatched here
     } else {
-      if (cout <= 3) {
-        VIE_CK(allow_smem(f_p5<T, R1, R2, 3>));
-        VIE_CK(launch_after(f_p5<T, R1, R2, 3>, grid, 256, smem(), st, A, xin, y, n, C, cout, He, Hm, wid, tw));
-      } else {
-        VIE_CK(allow_smem(f_p5<T, R1, R2, 6>));
-        VIE_CK(launch_after(f_p5<T, R1, R2, 6>, grid, 256, smem(), st, A, xin, y, n, C, cout, He, Hm, wid, tw));
-      }
-      VIE_CK(cudaGetLastError());
+      constexpr int NT = M <= 96 ? 64 : 256, rows = NT / R2;
+      const size_t sm = sizeof(V) * (M + rows * Fft2<T, R1, R2>::LS);
+      const dim3 grid((n * n + rows - 1) / rows, nrhs);
+      auto go = [&](auto kern) -> vie_status {
+        VIE_CK(allow_smem(kern));
+        VIE_CK(launch_after(kern, grid, NT, sm, st, A, xin, y, n, C, cout, He, Hm, wid, tw));
+        return VIE_OK;
+      };
+      return cout <= 3 ? go(f_p5<T, R1, R2, 3, NT>) : go(f_p5<T, R1, R2, 6, NT>);
+    }
+  }
+  // P1 and P2 in one kernel (FP32 up to M = 96).
+  static constexpr bool fused_xy = std::is_same<T, float>::value && M <= 96;
+  static vie_status p12(const E* x, V* B, int n, int C, int cin, int nrhs, const V* tw, cudaStream_t st) {
+    if constexpr (fused_xy) {
+      constexpr int NT = M / 2 * R2;
+      VIE_CK(allow_smem(f_p12<R1, R2>));
+      VIE_CK(launch_after(f_p12<R1, R2>, dim3(n, cin, nrhs), NT, sizeof(V) * (M + M * Fft2<T, R1, R2>::LS), st, x, B, C,
+                          tw));
       return VIE_OK;
+    } else {
+      return VIE_EINVAL;  // not dispatched here
     }
   }
 };
@@ -1732,8 +1807,12 @@ vie_status fast_pass(int pass, vie_problem* P, const KernelSet& K, const void* i
   const V* tw = Prec<T>::tw(P);
   const int cin = cin_of(K.mode), cout = cout_of(K.mode);
   switch (pass) {
-    case 1: return FP::p1((const typename IOT<T>::E*)in, A, n, C, cin, nrhs, tw, st);
-    case 2: return FP::template py<-1>(A, B, n, C, cin, nrhs, tw, st);
+    case 1:
+      if constexpr (FP::fused_xy) return FP::p12((const typename IOT<T>::E*)in, B, n, C, cin, nrhs, tw, st);
+      else return FP::p1((const typename IOT<T>::E*)in, A, n, C, cin, nrhs, tw, st);
+    case 2:
+      if constexpr (FP::fused_xy) return VIE_OK;  // done by pass 1
+      else return FP::template py<-1>(A, B, n, C, cin, nrhs, tw, st);
     case 3: {
       bool done = false;
       vie_status e = FP::p3v(P->p3_variant[Prec<T>::id][K.mode], B, n, C, Prec<T>::K(K), K.mode, nrhs,

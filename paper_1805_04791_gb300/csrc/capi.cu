@@ -36,10 +36,11 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 // Device memory comes from one pool per device, which keeps up to a thirty-second
 // of the device (kPoolShare) mapped when problems are destroyed: mapping and
 // unmapping cost about 1 ms a gigabyte each way, a fifth of a request at 192^3
-// (whole request 118 -> 99 ms at 192^3, 6.4 -> 5.1 ms at 64^3).  The pool gives everything unused back when one of the library's
-// allocations fails (which is then tried again), and when a problem is destroyed
-// while less than an eighth of the device is free.  Pools are made once per device and live
-// as long as the process; the CUDA calls on them are thread-safe and stream-ordered.
+// (whole request 118 -> 99 ms at 192^3, 6.4 -> 5.1 ms at 64^3).  The pool gives
+// everything unused back when one of the library's allocations fails (which is
+// then tried again), and when a problem is destroyed while less than an eighth of
+// the device is free.  Pools are made once per device and live as long as the
+// process; the CUDA calls on them are thread-safe and stream-ordered.
 static const int kPoolShare = 32, kPoolDevices = 64;
 static std::mutex g_pool_mutex;
 static cudaMemPool_t g_pool[kPoolDevices] = {nullptr};

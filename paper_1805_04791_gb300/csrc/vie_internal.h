@@ -204,12 +204,15 @@ inline cudaError_t allow_smem(K* kernel, bool max_carveout = false) {
 // Launch a kernel that starts with after_previous(): its blocks may take their
 // places while the last blocks of the stream's previous kernel still run
 // (programmatic stream serialization), so that the launch latency and the ramp of
-// a pass overlap the tail of the one before.  Only grids that fit the device about
-// at once gain by it (kLaunchAfterBlocks; whole request at 64^3 6.64 -> 6.21 ms,
-// solve at 32^3 1.19 -> 1.09 ms); blocks of a large grid that wait in the places of
-// its predecessor's last wave cost more than the latency (FP32 apply at 128^3 392 ->
-// 417 us), so those are launched plainly, where after_previous() returns at once.
-static const unsigned kLaunchAfterBlocks = 5 * 152;
+// a pass overlap the tail of the one before.  Only grids that leave most of the
+// device free gain by it (kLaunchAfterThreads: 448 threads an SM; FP32 apply at 32^3
+// 23.6 -> 21.7 us, at 48^3 42.5 -> 38.4, at 64^3 70.3 -> 61.4, solve at 32^3 1.19 -> 1.08 ms);
+// blocks that fill the device wait in the places of their predecessor's last wave
+// and cost more than the latency (32^3 with its z pass of 101 k threads launched so:
+// 33 us against 21.6; last pass at 96^3, 74 k threads: 223 against 213 us an apply;
+// every pass at 128^3: 417 against 392 us).  Those are launched plainly, where
+// after_previous() returns at once.
+static const unsigned long long kLaunchAfterThreads = 152 * 448;
 template <typename... P, typename... A>
 inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute at;
@@ -221,7 +224,9 @@ inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &at;
-  cfg.numAttrs = (unsigned long long)grid.x * grid.y * grid.z <= kLaunchAfterBlocks ? 1 : 0;
+  const unsigned long long threads =
+      (unsigned long long)grid.x * grid.y * grid.z * block.x * block.y * block.z;
+  cfg.numAttrs = threads <= kLaunchAfterThreads ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
