@@ -182,8 +182,14 @@ static void free_problem(vie_problem* P) {
   free_set(P->keval, st);
   cudaStreamSynchronize(st);
   for (cudaEvent_t e : P->prof.ev) cudaEventDestroy(e);
+  // kernels of a solve that ended early, on whatever stream, may still store to the
+  // pinned block; each is followed by one of these events or runs on cap_stream
+  if (P->cap_stream) cudaStreamSynchronize(P->cap_stream);
   for (cudaEvent_t e : P->arn_ev)
-    if (e) cudaEventDestroy(e);
+    if (e) {
+      cudaEventSynchronize(e);
+      cudaEventDestroy(e);
+    }
   if (P->arn_host) pinned_give(P->arn_host);
   for (cudaGraphExec_t g : P->graph_exec)
     if (g) cudaGraphExecDestroy(g);
