@@ -1251,8 +1251,8 @@ f_p3h(float2* __restrict__ B, int C, const float2* __restrict__ K, const float2*
     {
       const int vp = self_y ? (v == 0 ? 2 : 4) : v + 1;
       if (vp < 4)
-        prefetch_tile(tile_base(grp, vp) - l - (long long)(h * G) * cs + (long long)r * (NN / 2) * zs, NG * G, NN / 2, cs, zs,
-                      threadIdx.x, NTHR);
+        prefetch_tile(tile_base(grp, vp) - l - (long long)(h * G) * cs + (long long)r * (NN / 2) * zs, NG * G, NN / 2,
+                      cs, zs, threadIdx.x, NTHR);
     }
     __syncthreads();  // twiddle table written; the previous tile's readers of the lines are done
     // ---- forward: step 1 of every component into its line, step 2 from the lines
@@ -1561,7 +1561,8 @@ struct FastPath {
       return VIE_EINVAL;
     }
     VIE_CK(allow_smem(f_p3b<T, R1, R2, MODE, NP>));
-    VIE_CK(launch_after(f_p3b<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st, B, n, C, K, tw));
+    VIE_CK(launch_after(f_p3b<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st, B,
+                        n, C, K, tw));
     return VIE_OK;
   }
   template <int MODE, int NP>
@@ -1580,7 +1581,8 @@ struct FastPath {
     } else {
       if (sm > cap || sm > smem_optin()) return VIE_OK;
       VIE_CK(allow_smem(f_p3c<T, R1, R2, MODE, NP>));
-      VIE_CK(launch_after(f_p3c<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, B, n, C, K, tw));
+      VIE_CK(launch_after(f_p3c<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, B, n, C, K,
+                          tw));
       *done = true;
       return VIE_OK;
     }
@@ -1603,7 +1605,8 @@ struct FastPath {
       } else {
         if (sm > cap || sm > smem_optin()) return VIE_OK;
         VIE_CK(allow_smem(f_p3p<R1, R2, MODE, NP>));
-        VIE_CK(launch_after(f_p3p<R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
+        VIE_CK(launch_after(f_p3p<R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, (float2*)B, n,
+                            C, (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
       }
@@ -1638,7 +1641,8 @@ struct FastPath {
           if (per < 1) return VIE_OK;
           groups = std::min(groups, sms * per);
         }
-        VIE_CK(launch_after(f_p3t<R1, R2, MODE, NP>, dim3(groups, nrhs), NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
+        VIE_CK(launch_after(f_p3t<R1, R2, MODE, NP>, dim3(groups, nrhs), NTHR, sm, st, (float2*)B, n, C,
+                            (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
       }
@@ -1663,7 +1667,8 @@ struct FastPath {
         // the whole unified L1 as shared memory: MINB CTAs of ~75 KB per SM
         VIE_CK(allow_smem(kern, true));
         const int groups = (M / 2 + 1) * (NTX / 2);
-        VIE_CK(launch_after(kern, dim3(groups, nrhs), Cfg::NTHR, sm, st, (float2*)B, n, C, (const float2*)K, (const float2*)tw));
+        VIE_CK(launch_after(kern, dim3(groups, nrhs), Cfg::NTHR, sm, st, (float2*)B, n, C, (const float2*)K,
+                            (const float2*)tw));
         *done = true;
         return VIE_OK;
       }

@@ -207,9 +207,9 @@ __global__ void __launch_bounds__(256) k2_p1(const typename IOT<T>::E* __restric
 
 // P2 (S < 0) and P4 (S > 0), y-lines: block (nl, R1), lanes along kx.
 template <typename T, int RM, int S>
-__global__ void __launch_bounds__(sizeof(typename CT<T>::V) == 8 ? 384 : 192, 2) k2_py(const typename CT<T>::V* __restrict__ in, typename CT<T>::V* __restrict__ out,
-                                             int n, TwoPlan p, int LS, int C, int ncomp,
-                                             const typename CT<T>::V* __restrict__ twg) {
+__global__ void __launch_bounds__(sizeof(typename CT<T>::V) == 8 ? 384 : 192, 2)
+k2_py(const typename CT<T>::V* __restrict__ in, typename CT<T>::V* __restrict__ out, int n, TwoPlan p, int LS, int C,
+      int ncomp, const typename CT<T>::V* __restrict__ twg) {
   after_previous();
   typedef typename CT<T>::V V;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -612,16 +612,19 @@ vie_status two_line_pass(int pass, const TwoPlan& p, const TwoArgs& a, cudaStrea
   if (pass == 1) {
     const int rows = std::max(1, 256 / p.R1), LS = (p.R1 * p.PF) | 1;
     VIE_CK(allow_smem(k2_p1<T, RM>));
-    VIE_CK(launch_after(k2_p1<T, RM>, dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p, rows, LS), st, (const typename IOT<T>::E*)a.x, (V*)a.A, n, p, LS, a.C, tw));
+    VIE_CK(launch_after(k2_p1<T, RM>, dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p,
+                        rows, LS), st, (const typename IOT<T>::E*)a.x, (V*)a.A, n, p, LS, a.C, tw));
   } else {
     const int nl = sizeof(V) == 8 ? 16 : 8, LS = two_pitch(p, nl, sizeof(V)), nc = pass == 2 ? a.cin : a.cout;
     const dim3 grid((M + nl - 1) / nl, n, a.nrhs * nc), blk(nl, p.R1);
     if (pass == 2) {
       VIE_CK(allow_smem(k2_py<T, RM, -1>));
-      VIE_CK(launch_after(k2_py<T, RM, -1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.A, (V*)a.B, n, p, LS, a.C, nc, tw));
+      VIE_CK(launch_after(k2_py<T, RM, -1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.A, (V*)a.B, n, p, LS,
+                          a.C, nc, tw));
     } else {
       VIE_CK(allow_smem(k2_py<T, RM, 1>));
-      VIE_CK(launch_after(k2_py<T, RM, 1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.B, (V*)a.A, n, p, LS, a.C, nc, tw));
+      VIE_CK(launch_after(k2_py<T, RM, 1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.B, (V*)a.A, n, p, LS,
+                          a.C, nc, tw));
     }
   }
   VIE_CK(cudaGetLastError());
@@ -648,7 +651,8 @@ vie_status two_z_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   const dim3 grid(2 * ((p.M + nl - 1) / nl) * (p.M / 2 + 1), a.nrhs), blk(nl, h.R1, tz);
   auto go = [&](auto kern) -> vie_status {
     VIE_CK(allow_smem(kern));
-    VIE_CK(launch_after(kern, grid, blk, smem_of(nl), st, (V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K, (const V*)a.tw));
+    VIE_CK(launch_after(kern, grid, blk, smem_of(nl), st, (V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K,
+                        (const V*)a.tw));
     return VIE_OK;
   };
   if constexpr (std::is_same<T, df>::value) {  // the operator's kernel sets only
@@ -679,7 +683,9 @@ vie_status two_last_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   int rows = std::max(1, 256 / (p.R1 * tz));
   while (rows > 1 && two_smem<V>(p, (size_t)a.cout * rows, LS) > 100 * 1024) --rows;
   VIE_CK(allow_smem(k2_p5<T, RM>));
-  VIE_CK(launch_after(k2_p5<T, RM>, dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz), two_smem<V>(p, (size_t)a.cout * rows, LS), st, (const V*)a.A, (const E*)a.x, (E*)a.y, a.n, p, LS, a.C, a.cout, (const V*)a.He, (const V*)a.Hm, a.with_identity, (const V*)a.tw));
+  VIE_CK(launch_after(k2_p5<T, RM>, dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz), two_smem<V>(p,
+                      (size_t)a.cout * rows, LS), st, (const V*)a.A, (const E*)a.x, (E*)a.y, a.n, p, LS, a.C, a.cout,
+                      (const V*)a.He, (const V*)a.Hm, a.with_identity, (const V*)a.tw));
   return VIE_OK;
 }
 
