@@ -21,9 +21,11 @@ LIB = os.path.join(LIBDIR, "libvie_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", os.path.join(ROOT, "include")]
-SOURCES = ["capi.cu", "precompute.cu", "apply.cu", "krylov.cu", "apply_static.cu", "apply_fast_dw_256.cu"] + [
-    f"apply_fast_{m:03d}.cu" for m in (64, 96, 128, 192, 256, 384, 512)] + [
-    f"apply_two_{t}.cu" for t in ("f32_16", "f32_24", "f64_16", "f64_24", "df_16", "df_24", "df_z_16", "df_z_24")]
+# longest first, so that the last ones to start are short
+SOURCES = [f"apply_two_{u}.cu" for u in ("df_z_24", "df_z_16", "f32_24", "f64_24", "df_24", "df_16")] + [
+    f"apply_fast_{m:03d}.cu" for m in (512, 256, 384, 128, 192)] + [
+    "apply.cu", "apply_two_f32_16.cu", "apply_two_f64_16.cu", "apply_fast_096.cu", "apply_fast_064.cu",
+    "apply_fast_dw_256.cu", "precompute.cu", "krylov.cu", "capi.cu", "apply_static.cu"]
 
 
 def nvcc() -> str:
