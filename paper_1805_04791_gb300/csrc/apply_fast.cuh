@@ -1538,7 +1538,7 @@ struct FastPath {
   typedef typename IOT<T>::E E;
   static vie_status p1(const E* x, V* A, int n, int C, int cin, int nrhs, const V* tw, cudaStream_t st) {
     VIE_CK(allow_smem(f_p1<T, R1, R2>));
-    VIE_CK(launch_after(f_p1<T, R1, R2>, dim3((n * n + L - 1) / L, cin, nrhs), 256, smem(), st, x, A, n, C, tw));
+    VIE_CK(launch_after<kOverlap<T>>(f_p1<T, R1, R2>, dim3((n * n + L - 1) / L, cin, nrhs), 256, smem(), st, x, A, n, C, tw));
     return VIE_OK;
   }
   template <int S>
@@ -1547,7 +1547,7 @@ struct FastPath {
       return VIE_EINVAL;  // not dispatched here
     } else {
       VIE_CK(allow_smem(f_py<T, R1, R2, S>));
-      VIE_CK(launch_after(f_py<T, R1, R2, S>, dim3(M / L, n, nrhs * nc), 256, smem(), st, in, out, n, C, nc, tw));
+      VIE_CK(launch_after<kOverlap<T>>(f_py<T, R1, R2, S>, dim3(M / L, n, nrhs * nc), 256, smem(), st, in, out, n, C, nc, tw));
       return VIE_OK;
     }
   }
@@ -1561,7 +1561,7 @@ struct FastPath {
       return VIE_EINVAL;
     }
     VIE_CK(allow_smem(f_p3b<T, R1, R2, MODE, NP>));
-    VIE_CK(launch_after(f_p3b<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st, B,
+    VIE_CK(launch_after<kOverlap<T>>(f_p3b<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2) * 4, nrhs), NP * R2 * CMAX, sm, st, B,
                         n, C, K, tw));
     return VIE_OK;
   }
@@ -1581,7 +1581,7 @@ struct FastPath {
     } else {
       if (sm > cap || sm > smem_optin()) return VIE_OK;
       VIE_CK(allow_smem(f_p3c<T, R1, R2, MODE, NP>));
-      VIE_CK(launch_after(f_p3c<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, B, n, C, K,
+      VIE_CK(launch_after<kOverlap<T>>(f_p3c<T, R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, B, n, C, K,
                           tw));
       *done = true;
       return VIE_OK;
@@ -1605,7 +1605,7 @@ struct FastPath {
       } else {
         if (sm > cap || sm > smem_optin()) return VIE_OK;
         VIE_CK(allow_smem(f_p3p<R1, R2, MODE, NP>));
-        VIE_CK(launch_after(f_p3p<R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, (float2*)B, n,
+        VIE_CK(launch_after<kOverlap<T>>(f_p3p<R1, R2, MODE, NP>, dim3((M / 2 + 1) * (NTX / 2), nrhs), NTHR, sm, st, (float2*)B, n,
                             C, (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
@@ -1641,7 +1641,7 @@ struct FastPath {
           if (per < 1) return VIE_OK;
           groups = std::min(groups, sms * per);
         }
-        VIE_CK(launch_after(f_p3t<R1, R2, MODE, NP>, dim3(groups, nrhs), NTHR, sm, st, (float2*)B, n, C,
+        VIE_CK(launch_after<kOverlap<T>>(f_p3t<R1, R2, MODE, NP>, dim3(groups, nrhs), NTHR, sm, st, (float2*)B, n, C,
                             (const float2*)K, (const float2*)tw));
         *done = true;
         return VIE_OK;
@@ -1667,7 +1667,7 @@ struct FastPath {
         // the whole unified L1 as shared memory: MINB CTAs of ~75 KB per SM
         VIE_CK(allow_smem(kern, true));
         const int groups = (M / 2 + 1) * (NTX / 2);
-        VIE_CK(launch_after(kern, dim3(groups, nrhs), Cfg::NTHR, sm, st, (float2*)B, n, C, (const float2*)K,
+        VIE_CK(launch_after<kOverlap<T>>(kern, dim3(groups, nrhs), Cfg::NTHR, sm, st, (float2*)B, n, C, (const float2*)K,
                             (const float2*)tw));
         *done = true;
         return VIE_OK;
@@ -1782,7 +1782,7 @@ struct FastPath {
       const dim3 grid((n * n + rows - 1) / rows, nrhs);
       auto go = [&](auto kern) -> vie_status {
         VIE_CK(allow_smem(kern));
-        VIE_CK(launch_after(kern, grid, NT, sm, st, A, xin, y, n, C, cout, He, Hm, wid, tw));
+        VIE_CK(launch_after<kOverlap<T>>(kern, grid, NT, sm, st, A, xin, y, n, C, cout, He, Hm, wid, tw));
         return VIE_OK;
       };
       return cout <= 3 ? go(f_p5<T, R1, R2, 3, NT>) : go(f_p5<T, R1, R2, 6, NT>);
@@ -1794,7 +1794,7 @@ struct FastPath {
     if constexpr (fused_xy) {
       constexpr int NT = M / 2 * R2;
       VIE_CK(allow_smem(f_p12<R1, R2>));
-      VIE_CK(launch_after(f_p12<R1, R2>, dim3(n, cin, nrhs), NT, sizeof(V) * (M + M * Fft2<T, R1, R2>::LS), st, x, B, C,
+      VIE_CK(launch_after<kOverlap<T>>(f_p12<R1, R2>, dim3(n, cin, nrhs), NT, sizeof(V) * (M + M * Fft2<T, R1, R2>::LS), st, x, B, C,
                           tw));
       return VIE_OK;
     } else {

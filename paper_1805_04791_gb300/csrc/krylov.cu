@@ -980,8 +980,8 @@ static vie_status gmres_cycle(vie_problem* P, Group& g, const std::vector<double
       r0 = r1;
     }
     for (int pass = 0; pass < 2; ++pass) {
-      VIE_CK(launch_after(k_arn_dots<TB>, dotg, kRedThreads, 0, ss, V, ldi, j, L, A, pass));
-      VIE_CK(launch_after(k_arn_axpy<TB>, redg, kRedThreads, 0, ss, V, ldi, j, L, A, pass,
+      VIE_CK(launch_after<kOverlap<TB>>(k_arn_dots<TB>, dotg, kRedThreads, 0, ss, V, ldi, j, L, A, pass));
+      VIE_CK(launch_after<kOverlap<TB>>(k_arn_axpy<TB>, redg, kRedThreads, 0, ss, V, ldi, j, L, A, pass,
                           pass == 1 ? mirror + (size_t)(j % kArnSlots) * nb : nullptr));
     }
     // inside a stream capture the record must be External to become an event-record

@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/vie.h"
@@ -213,7 +214,11 @@ inline cudaError_t allow_smem(K* kernel, bool max_carveout = false) {
 // every pass at 128^3: 417 against 392 us).  Those are launched plainly, where
 // after_previous() returns at once.
 static const unsigned long long kLaunchAfterThreads = 152 * 448;
-template <typename... P, typename... A>
+// FP64 passes and reductions are launched plainly too: bound by the FP64 pipe, they
+// are long for their grids and lose by it (FP64 apply at 32^3 142 us, 197 launched so;
+// double-word 70 us, 59 launched so).
+template <typename T> constexpr bool kOverlap = !std::is_same<T, double>::value && !std::is_same<T, double2>::value;
+template <bool OVERLAP, typename... P, typename... A>
 inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -226,7 +231,7 @@ inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_
   cfg.attrs = &at;
   const unsigned long long threads =
       (unsigned long long)grid.x * grid.y * grid.z * block.x * block.y * block.z;
-  cfg.numAttrs = threads <= kLaunchAfterThreads ? 1 : 0;
+  cfg.numAttrs = OVERLAP && threads <= kLaunchAfterThreads ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 

@@ -612,18 +612,18 @@ vie_status two_line_pass(int pass, const TwoPlan& p, const TwoArgs& a, cudaStrea
   if (pass == 1) {
     const int rows = std::max(1, 256 / p.R1), LS = (p.R1 * p.PF) | 1;
     VIE_CK(allow_smem(k2_p1<T, RM>));
-    VIE_CK(launch_after(k2_p1<T, RM>, dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p,
+    VIE_CK(launch_after<kOverlap<T>>(k2_p1<T, RM>, dim3((n * n + rows - 1) / rows, a.cin, a.nrhs), dim3(p.R1, rows), two_smem<V>(p,
                         rows, LS), st, (const typename IOT<T>::E*)a.x, (V*)a.A, n, p, LS, a.C, tw));
   } else {
     const int nl = sizeof(V) == 8 ? 16 : 8, LS = two_pitch(p, nl, sizeof(V)), nc = pass == 2 ? a.cin : a.cout;
     const dim3 grid((M + nl - 1) / nl, n, a.nrhs * nc), blk(nl, p.R1);
     if (pass == 2) {
       VIE_CK(allow_smem(k2_py<T, RM, -1>));
-      VIE_CK(launch_after(k2_py<T, RM, -1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.A, (V*)a.B, n, p, LS,
+      VIE_CK(launch_after<kOverlap<T>>(k2_py<T, RM, -1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.A, (V*)a.B, n, p, LS,
                           a.C, nc, tw));
     } else {
       VIE_CK(allow_smem(k2_py<T, RM, 1>));
-      VIE_CK(launch_after(k2_py<T, RM, 1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.B, (V*)a.A, n, p, LS,
+      VIE_CK(launch_after<kOverlap<T>>(k2_py<T, RM, 1>, grid, blk, two_smem<V>(p, nl, LS), st, (const V*)a.B, (V*)a.A, n, p, LS,
                           a.C, nc, tw));
     }
   }
@@ -651,7 +651,7 @@ vie_status two_z_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   const dim3 grid(2 * ((p.M + nl - 1) / nl) * (p.M / 2 + 1), a.nrhs), blk(nl, h.R1, tz);
   auto go = [&](auto kern) -> vie_status {
     VIE_CK(allow_smem(kern));
-    VIE_CK(launch_after(kern, grid, blk, smem_of(nl), st, (V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K,
+    VIE_CK(launch_after<kOverlap<T>>(kern, grid, blk, smem_of(nl), st, (V*)a.B, a.n, h, LS, a.C, a.mode, (const V*)a.K,
                         (const V*)a.tw));
     return VIE_OK;
   };
@@ -683,7 +683,7 @@ vie_status two_last_pass(const TwoPlan& p, const TwoArgs& a, cudaStream_t st) {
   int rows = std::max(1, 256 / (p.R1 * tz));
   while (rows > 1 && two_smem<V>(p, (size_t)a.cout * rows, LS) > 100 * 1024) --rows;
   VIE_CK(allow_smem(k2_p5<T, RM>));
-  VIE_CK(launch_after(k2_p5<T, RM>, dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz), two_smem<V>(p,
+  VIE_CK(launch_after<kOverlap<T>>(k2_p5<T, RM>, dim3((a.n * a.n + rows - 1) / rows, a.nrhs), dim3(p.R1, rows, tz), two_smem<V>(p,
                       (size_t)a.cout * rows, LS), st, (const V*)a.A, (const E*)a.x, (E*)a.y, a.n, p, LS, a.C, a.cout,
                       (const V*)a.He, (const V*)a.Hm, a.with_identity, (const V*)a.tw));
   return VIE_OK;
