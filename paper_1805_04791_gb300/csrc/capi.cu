@@ -175,6 +175,11 @@ static void free_set(KernelSet& k, cudaStream_t st) {
 static void free_problem(vie_problem* P) {
   if (!P) return;
   cudaStream_t st = P->stream;
+  // steps of a solve, on whatever stream, write to the buffers and to the pinned block;
+  // each is followed by one of these events or runs on cap_stream
+  if (P->cap_stream) cudaStreamSynchronize(P->cap_stream);
+  for (cudaEvent_t e : P->arn_ev)
+    if (e) cudaEventSynchronize(e);
   void* ptrs[] = {P->tw64, P->tw32, P->He64, P->He32, P->Hm64, P->Hm32, P->twdf, P->Hedf, P->Hmdf,
                   P->base_oct, P->ws.buf, P->ks.buf, P->dflag};
   for (void* q : ptrs) dfree(q, st);
@@ -182,14 +187,8 @@ static void free_problem(vie_problem* P) {
   free_set(P->keval, st);
   cudaStreamSynchronize(st);
   for (cudaEvent_t e : P->prof.ev) cudaEventDestroy(e);
-  // kernels of a solve that ended early, on whatever stream, may still store to the
-  // pinned block; each is followed by one of these events or runs on cap_stream
-  if (P->cap_stream) cudaStreamSynchronize(P->cap_stream);
   for (cudaEvent_t e : P->arn_ev)
-    if (e) {
-      cudaEventSynchronize(e);
-      cudaEventDestroy(e);
-    }
+    if (e) cudaEventDestroy(e);
   if (P->arn_host) pinned_give(P->arn_host);
   for (cudaGraphExec_t g : P->graph_exec)
     if (g) cudaGraphExecDestroy(g);

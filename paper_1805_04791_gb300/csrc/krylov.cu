@@ -1418,8 +1418,8 @@ static double fp32_apply_error(const vie_problem* P, double dn) {
   return (14.0 * u * 3.0 * std::log2(M) + 4.0 * u) * P->opnorm * dn * 1.01;
 }
 
-vie_status run_solve(vie_problem* P, const void* rhs, void* Jv, const vie_solve_opts* opt, vie_solve_info* info,
-                     cudaStream_t st) {
+static vie_status solve_steps(vie_problem* P, const void* rhs, void* Jv, const vie_solve_opts* opt,
+                              vie_solve_info* info, cudaStream_t st) {
   const auto t0 = std::chrono::steady_clock::now();
   const long long L = (long long)P->ncomp * P->n * P->n * P->n;
   const int m = opt->restart;
@@ -1569,6 +1569,20 @@ vie_status run_solve(vie_problem* P, const void* rhs, void* Jv, const vie_solve_
   if (info) *info = inf;
   if (final_status == VIE_ENOCONV) set_error("GMRES did not reach the tolerance within the iteration limits");
   return final_status;
+}
+
+vie_status run_solve(vie_problem* P, const void* rhs, void* Jv, const vie_solve_opts* opt, vie_solve_info* info,
+                     cudaStream_t st) {
+  const vie_status s = solve_steps(P, rhs, Jv, opt, info, st);
+  // A solve that ended early may have steps running on st or on the graphs' stream,
+  // which st has not waited for; they write to the workspaces and to the pinned block.
+  // None may outlive the call: the next call, or the destruction of the problem on
+  // another stream, takes those for unused.
+  if (s != VIE_OK && s != VIE_ENOCONV) {
+    if (P->cap_stream) cudaStreamSynchronize(P->cap_stream);
+    cudaStreamSynchronize(st);
+  }
+  return s;
 }
 
 }  // namespace vie

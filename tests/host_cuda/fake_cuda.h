@@ -1,0 +1,31 @@
+// A CUDA runtime that runs nothing: device memory is host memory, kernels and copies to
+// the device do nothing, and every call that matters to ordering or memory is recorded.
+// Host code linked against it (instead of the CUDA runtime) can be checked without a
+// GPU, with any call made to fail.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+#include <vector>
+
+namespace fake {
+
+enum Op { LAUNCH, COPY, MEMSET, RECORD, FREE, STREAM_SYNC, EVENT_SYNC, STREAM_WAIT };
+
+struct Call {
+  Op op;
+  uintptr_t stream;  // of LAUNCH, COPY, MEMSET, RECORD, FREE, STREAM_SYNC, STREAM_WAIT
+  uintptr_t event;   // of RECORD, EVENT_SYNC, STREAM_WAIT
+};
+
+struct State {
+  std::vector<Call> log;
+  long work = 0;         // launches, copies, memsets and event records so far
+  long fail_at = -1;     // the work call (counted from `work`) that fails; -1: none
+  bool ones = false;     // copies of reduction results to the host read as 1.0
+  size_t live = 0, high = 0;    // device bytes allocated now, and at most
+  size_t total = 1ull << 38;    // bytes of the device
+};
+State& state();
+
+}  // namespace fake
