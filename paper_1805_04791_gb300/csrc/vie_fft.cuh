@@ -215,22 +215,31 @@ __device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& h, float2& 
 }
 // The complex operations below are bound by the FP32 pipes (a packed f32x2
 // instruction takes both lanes' slots), so each is written for the fewest of
-// them; no lane needs a runtime negation, signs being factors of an FMA.
+// them that keep a transform's error below that of the algorithms above; no lane
+// needs a runtime negation, signs being factors of an FMA.  What counts is how many
+// roundings of the size of a low word (u^2 of the result) an operation makes.  The last
+// low sum of each, e, is used rounded for the high word only: with d = the part of
+// it that the high word took (exact), the low word is formed as (first term of e - d) +
+// rest, where the subtraction is nearly always exact, so that e's rounding is not
+// in the result, for one instruction more than a Fast2Sum.
+// RMS errors of transforms of 48 to 440 points: 2.6 - 3.6e-15 of the norm, against
+// 2.8 - 3.8e-15 with the algorithms above throughout and 3.1 - 4.4e-15 with Fast2Sums
+// here (11 and 19 instructions); of convolutions 4.2 - 5.0, 4.5 - 5.5 and 5.1 - 6.1e-15.
+// Double-word apply, Helmholtz 96^3: 1.18 ms, 1.11 with those Fast2Sums.
 //
 // Sum per lane, x + c y with c = +-1 per lane: TwoSum of the high words, the low
-// words added to its error, one Fast2Sum (11 instructions; "SloppyDWPlusDW" of
-// Joldes, Muller and Popescu).  Its error is about 2u^2 (|x| + |y|); the 20
-// instructions of "AccurateDWPlusDW" bound it by 3u^2 |x + y|, which differs only
-// where the sum cancels, and a butterfly's other output then carries the larger
-// part: in a transform the errors are those of the norm either way.
-// Double-word apply, Helmholtz 96^3: 2.22 -> 1.49 ms with dw_addc and dw_dot2.
+// words added to its error (12 instructions; AccurateDWPlusDW takes 20 and makes
+// about as many such roundings).  Its error is about 2u^2 (|x| + |y|) where the published
+// bound is 3u^2 |x + y|: a sum that cancels is less exact than there, relative to
+// itself, not relative to the data.
 __device__ __forceinline__ cdf dw_addc(float2 xh, float2 xl, float2 yh, float2 yl, float2 c) {
   const float2 s = fma2(yh, c, xh);
   const float2 nb = sub2(xh, s);
   const float2 t = add2(sub2(xh, add2(s, nb)), fma2(yh, c, nb));
-  const float2 e = add2(t, fma2(yl, c, xl));
+  const float2 v = fma2(yl, c, xl);
   cdf r;
-  fast_two_sum2(s, e, r.h, r.l);
+  r.h = add2(s, add2(t, v));
+  r.l = add2(sub2(t, sub2(r.h, s)), v);
   return r;
 }
 // DWTimesDW3 per lane: (xh, xl) (yh, yl)
@@ -243,23 +252,24 @@ __device__ __forceinline__ cdf dw_mul2(float2 xh, float2 xl, float2 yh, float2 y
   fast_two_sum2(ch, add2(cl1, cl2), r.h, r.l);
   return r;
 }
-// a w + swap(a) v per lane with one normalisation (19 instructions; two products
-// and a sum, each normalised, take 38): the high products with their FMA-exact
-// errors, TwoSum of the two, every first-order low term added to its error, one
-// Fast2Sum.  nw and nv are -w and -v of the high words: the products are formed
-// negated so that their errors are plain FMAs.
+// a w + swap(a) v per lane with one normalisation (23 instructions; two DWTimesDW3
+// and a sum take 38): the high products with their FMA-exact errors, TwoSum of the
+// two, the first-order low terms of each product added to its error, the two low
+// sums and TwoSum's error added, both roundings of that recovered (the first
+// as Fast2Sum does).  Left out are the products of two low words, u^2 / 4 at most
+// and 0.16 u^2 on average.  nw and nv are -w and -v of the high words: the products
+// are formed negated so that their errors are plain FMAs.
 __device__ __forceinline__ cdf dw_dot2(cdf a, float2 wh, float2 nwh, float2 wl, float2 vh, float2 nvh, float2 vl) {
   const float2 bh = swp(a.h), bl = swp(a.l);
   const float2 np = mul2(a.h, nwh), nq = mul2(bh, nvh);
-  float2 e = fma2(a.l, wh, fma2(a.h, wh, np)), g = fma2(bl, vh, fma2(bh, vh, nq));
-  e = fma2(a.h, wl, e);
-  g = fma2(bh, vl, g);
+  const float2 e = fma2(a.h, wl, fma2(a.l, wh, fma2(a.h, wh, np)));
+  const float2 g = fma2(bh, vl, fma2(bl, vh, fma2(bh, vh, nq)));
   float2 ns, nt;
   two_sum2(np, nq, ns, nt);
-  e = sub2(add2(e, g), nt);
+  const float2 f = add2(e, g);
   cdf r;
-  r.h = sub2(e, ns);
-  r.l = sub2(e, add2(r.h, ns));
+  r.h = sub2(sub2(f, nt), ns);
+  r.l = add2(sub2(sub2(f, add2(r.h, ns)), nt), sub2(g, sub2(f, e)));
   return r;
 }
 __device__ __forceinline__ cdf operator+(cdf a, cdf b) { return dw_addc(a.h, a.l, b.h, b.l, make_float2(1.f, 1.f)); }
@@ -282,7 +292,7 @@ __device__ __forceinline__ cdf rot(cdf a, df c, df s) {
   return dw_dot2(a, make_float2(c.hi, c.hi), make_float2(-c.hi, -c.hi), make_float2(c.lo, c.lo),
                  make_float2(-s.hi, s.hi), make_float2(s.hi, -s.hi), make_float2(-s.lo, s.lo));
 }
-// c + s a with one normalisation (15 instructions), as dw_dot2
+// c + s a with one normalisation (16 instructions), as dw_dot2
 __device__ __forceinline__ cdf cfma(df s, cdf a, cdf c) {
   const float2 sh = make_float2(s.hi, s.hi), sl = make_float2(s.lo, s.lo);
   const float2 np = mul2(a.h, make_float2(-s.hi, -s.hi));
@@ -290,9 +300,10 @@ __device__ __forceinline__ cdf cfma(df s, cdf a, cdf c) {
   const float2 t0 = sub2(c.h, np);  // c + s a rounded; then TwoSum's error with b = -np
   const float2 nb = sub2(c.h, t0);
   const float2 t = add2(sub2(c.h, add2(t0, nb)), sub2(nb, np));
-  const float2 e = add2(add2(g, c.l), t);
+  const float2 f = add2(g, c.l);
   cdf r;
-  fast_two_sum2(t0, e, r.h, r.l);
+  r.h = add2(t0, add2(f, t));
+  r.l = add2(sub2(t, sub2(r.h, t0)), f);
   return r;
 }
 __device__ __forceinline__ cdf vneg(cdf a) {
@@ -334,7 +345,7 @@ __device__ __forceinline__ double2 from_v<df>(cdf v) {
 // double-word path adds its a + b + c to the FP64 x in FP64: the identity part,
 // usually the larger, keeps all its bits (rounding x and the three sums to 48
 // bits was most of the apply's error, 1.8e-15 against 64 bits at Helmholtz 96^3 and
-// 5e-16 without), and x needs no conversion.
+// 4.5e-16 without), and x needs no conversion.
 template <typename T>
 __device__ __forceinline__ typename IOT<T>::E add_id(typename IOT<T>::E x, typename CT<T>::V a, typename CT<T>::V b,
                                                      typename CT<T>::V c) {
