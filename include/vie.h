@@ -46,8 +46,9 @@
  *                       (see vie_tune), bypassing the process-wide tuning
  *                       cache; shapes k does not fit return VIE_EINVAL.
  * - VIE_TUNE=0          vie_tune takes the first applicable variant untimed.
- * - VIE_GENERIC_FFT     (set to any value) the generic shared-memory kernels
- *                       run at every size, also where register-resident ones exist.
+ * - VIE_GENERIC_FFT     (set to any value) the generic shared-memory Stockham
+ *                       kernels run at every size, also where register-resident or
+ *                       two-step ones exist.
  * - VIE_GROUP_MAX=g     batched solves use lockstep groups of at most g
  *                       right-hand sides (default: from free device memory, <= 64).
  * - VIE_RESIDUAL_FP64=1 mixed solves compute their residuals with the native

@@ -319,10 +319,13 @@ struct FastSel {
 // per line: 2n when the convolution grid is 2n, else 0 (no fast kernels).
 static int fast_grid(const vie_problem* P) { return P->nk == P->n ? 2 * P->n : 0; }
 
+// VIE_GENERIC_FFT: the shared-memory Stockham kernels at every size.
+static bool generic_forced() { return getenv("VIE_GENERIC_FFT") != nullptr; }
+
 static FastSel fast_select(int M, int mode, int with_identity) {
   FastSel f;
   if (M != 64 && M != 96 && M != 128 && M != 192 && M != 256 && M != 384 && M != 512) return f;
-  if (getenv("VIE_GENERIC_FFT")) return f;
+  if (generic_forced()) return f;
   const int cin = cin_of(mode), cout = cout_of(mode);
   f.p1 = true;
   f.py = true;
@@ -483,7 +486,7 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
   }
   if (p3v == kP3Generic) fs.p3 = false;
   TwoPlan tp;
-  const bool two = make_two_plan(M, &tp);
+  const bool two = make_two_plan(M, &tp) && !generic_forced();
   if (Prec<T>::id == VIE_FP64 && fp64_two_y(M)) {
     fs.py = false;
     if (fp64_two_last(M)) fs.p5 = false;
