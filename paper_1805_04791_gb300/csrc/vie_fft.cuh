@@ -225,7 +225,8 @@ __device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& h, float2& 
 // RMS errors of transforms of 48 to 440 points: 2.6 - 3.6e-15 of the norm, against
 // 2.8 - 3.8e-15 with the algorithms above throughout and 3.1 - 4.4e-15 with Fast2Sums
 // here (11 and 19 instructions); of convolutions 4.2 - 5.0, 4.5 - 5.5 and 5.1 - 6.1e-15.
-// Double-word apply, Helmholtz 96^3: 1.18 ms, 1.11 with those Fast2Sums.
+// Double-word apply, Helmholtz 96^3: 1.17 ms; 1.84 with the algorithms above throughout,
+// 1.11 with those Fast2Sums.
 //
 // Sum per lane, x + c y with c = +-1 per lane: TwoSum of the high words, the low
 // words added to its error (12 instructions; AccurateDWPlusDW takes 20 and makes
@@ -256,8 +257,8 @@ __device__ __forceinline__ cdf dw_mul2(float2 xh, float2 xl, float2 yh, float2 y
 // and a sum take 38): the high products with their FMA-exact errors, TwoSum of the
 // two, the first-order low terms of each product added to its error, the two low
 // sums and TwoSum's error added, both roundings of that recovered (the first
-// as Fast2Sum does).  Left out are the products of two low words, u^2 / 4 at most
-// and 0.16 u^2 on average.  nw and nv are -w and -v of the high words: the products
+// as Fast2Sum does).  Left out are the products of two low words, u^2 at most and
+// 0.17 u^2 on average.  nw and nv are -w and -v of the high words: the products
 // are formed negated so that their errors are plain FMAs.
 __device__ __forceinline__ cdf dw_dot2(cdf a, float2 wh, float2 nwh, float2 wl, float2 vh, float2 nvh, float2 vl) {
   const float2 bh = swp(a.h), bl = swp(a.l);
