@@ -26,7 +26,8 @@
  *   and Maxwell with mu = I; c = 6 ([J; M]) for Maxwell with mu.
  * - "device" pointers are CUDA device memory of the current device; the
  *   caller owns every pointer it passes in (the library never frees them).
- *   The library owns everything it allocates, from create until destroy.
+ *   The library owns everything it allocates, from create until destroy, and
+ *   keeps a bounded part of it for the next problem (vie_release_memory).
  * - stream is a cudaStream_t (NULL = legacy default stream).  Calls enqueue
  *   work on it and return without synchronising unless stated otherwise.
  * - No exception crosses the ABI; every call returns a vie_status and, on
@@ -34,8 +35,9 @@
  * - A problem handle is not thread-safe; distinct handles may be used from
  *   different threads on different streams.  Calls on one handle must be
  *   ordered (one stream, or streams the caller synchronises).  Device memory
- *   is allocated stream-ordered (cudaMallocAsync) on the stream of the call,
- *   so calls on other handles and streams are never serialised by it; the
+ *   is allocated stream-ordered on the stream of the call, from one memory pool of
+ *   the library per device, so calls on other handles and streams are never
+ *   serialised by it; the
  *   stream given to vie_problem_create must stay valid until
  *   vie_problem_destroy, which frees on it.
  *
@@ -248,8 +250,18 @@ vie_status vie_eval_scattered(vie_problem* P, const void* J, void* field_out, in
 size_t vie_problem_bytes(int kind, int n, int nrhs, int restart, int has_mu);
 
 /* Release every allocation of the handle, stream-ordered on the stream the
- * handle was created with, and wait for that stream. */
+ * handle was created with, and wait for that stream.  The memory goes back to the
+ * library's pool, which keeps up to a thirty-second of the device mapped for the next
+ * problem; all of it goes back to the device when an allocation of the library fails
+ * (which is then tried again), when less than an eighth of the device is free, and by
+ * vie_release_memory.  Up to sixteen pinned host blocks of 64 KiB are kept as well. */
 vie_status vie_problem_destroy(vie_problem* P);
+
+/* Give back what the library keeps for the next problem: the device memory of the
+ * current device's pool that no handle uses, and the kept pinned blocks.  Handles and
+ * calls in flight are not affected; the next problem maps its memory anew (about 1 ms
+ * a gigabyte).  For processes whose other allocators need the memory. */
+vie_status vie_release_memory(void);
 
 /* Autotune the z-pass schedule of vie_apply at this precision by timing every
  * applicable variant on this device; the choice is kept in the handle and

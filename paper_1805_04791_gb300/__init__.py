@@ -31,7 +31,7 @@ STATUS_NAMES = {0: "VIE_OK", 1: "VIE_EINVAL", 2: "VIE_ENOMEM", 3: "VIE_ECUDA", 4
 
 EXPORTED = ("vie_problem_create", "vie_problem_ncomp", "vie_apply", "vie_rhs_plane_wave", "vie_solve",
             "vie_eval_scattered", "vie_problem_bytes", "vie_problem_destroy", "vie_last_error",
-            "vie_profile_begin", "vie_profile_end", "vie_tune", "vie_apply_static")
+            "vie_profile_begin", "vie_profile_end", "vie_tune", "vie_apply_static", "vie_release_memory")
 
 
 class VieError(RuntimeError):
@@ -92,6 +92,8 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.vie_apply_static.restype = c_int
     lib.vie_tune.argtypes = [vp, c_int, ctypes.POINTER(c_int), vp]
     lib.vie_tune.restype = c_int
+    lib.vie_release_memory.argtypes = []
+    lib.vie_release_memory.restype = c_int
     lib.vie_last_error.argtypes = []
     lib.vie_last_error.restype = ctypes.c_char_p
     _lib = lib
@@ -221,6 +223,11 @@ def vie_problem_bytes(kind: int, n: int, nrhs: int, restart: int, has_mu: int) -
 def vie_problem_destroy(P):
     _SHAPES.pop(_key(P), None)
     return _check(load().vie_problem_destroy(P))
+
+
+def vie_release_memory():
+    """Give back the device memory and pinned blocks the library keeps for the next problem."""
+    return _check(load().vie_release_memory())
 
 
 def vie_profile_begin(P, cap: int):

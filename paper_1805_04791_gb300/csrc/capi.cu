@@ -38,8 +38,9 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 // unmapping cost about 1 ms a gigabyte each way, a fifth of a request at 192^3
 // (whole request 118 -> 99 ms at 192^3, 6.4 -> 5.1 ms at 64^3).  The pool gives
 // everything unused back when one of the library's allocations fails (which is
-// then tried again), and when a problem is destroyed while less than an eighth of
-// the device is free.  Pools are made once per device and live as long as the
+// then tried again), when a problem is destroyed while less than an eighth of
+// the device is free, and when the caller asks for it (vie_release_memory): another
+// allocator in the process cannot take what the pool keeps.  Pools are made once per device and live as long as the
 // process; the CUDA calls on them are thread-safe and stream-ordered.
 static const int kPoolShare = 32, kPoolDevices = 64;
 static std::mutex g_pool_mutex;
@@ -425,6 +426,18 @@ vie_status vie_profile_end(vie_problem* P, double* ms, int nslots, int* count) {
 
 vie_status vie_problem_destroy(vie_problem* P) {
   free_problem(P);
+  return VIE_OK;
+}
+
+vie_status vie_release_memory(void) {
+  std::vector<void*> blocks;
+  {
+    std::lock_guard<std::mutex> g(g_pool_mutex);
+    blocks.swap(g_pinned);
+  }
+  for (void* p : blocks) cudaFreeHost(p);
+  cudaMemPool_t pool = device_pool();
+  if (pool) VIE_CK(cudaMemPoolTrimTo(pool, 0));
   return VIE_OK;
 }
 

@@ -33,7 +33,8 @@ static cudaError_t note(Op op, cudaStream_t st, uintptr_t ev = 0) {
 }
 static cudaError_t take(void** p, size_t bytes) {
   State& s = state();
-  if (s.live + bytes > s.total) {
+  if (s.live + s.kept + s.foreign + bytes > s.total) {
+    ++s.refused;
     g_last = cudaErrorMemoryAllocation;
     return g_last;
   }
@@ -101,31 +102,41 @@ E cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) { ret
 E cudaMallocAsync(void** p, size_t n, cudaStream_t) { return take(p, n); }
 E cudaFreeAsync(void* p, cudaStream_t st) {
   state().live -= g_sizes[p];
+  state().kept += g_sizes[p];
   g_sizes.erase(p);
   free(p);
   return note(FREE, st);
 }
 E cudaMallocHost(void** p, size_t n) {
   *p = calloc(1, n);
+  ++state().host_blocks;
   return cudaSuccess;
 }
 E cudaFreeHost(void* p) {
+  --state().host_blocks;
   free(p);
   return cudaSuccess;
 }
 E cudaMemGetInfo(size_t* f, size_t* t) {
   *t = state().total;
-  *f = state().total - state().live;
+  *f = state().total - state().live - state().kept - state().foreign;
   return cudaSuccess;
 }
 E cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*) { return handle(p); }
 E cudaMemPoolDestroy(cudaMemPool_t) { return cudaSuccess; }
-E cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr, void* v) {
-  *(uint64_t*)v = 0;
+E cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr a, void* v) {
+  *(uint64_t*)v = state().live + (a == cudaMemPoolAttrReservedMemCurrent ? state().kept : 0);
   return cudaSuccess;
 }
-E cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { return cudaSuccess; }
-E cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaSuccess; }
+E cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr a, void* v) {
+  if (a == cudaMemPoolAttrReleaseThreshold) state().threshold = *(uint64_t*)v;
+  return cudaSuccess;
+}
+E cudaMemPoolTrimTo(cudaMemPool_t, size_t) {
+  if (state().kept) ++state().trims;
+  state().kept = 0;
+  return cudaSuccess;
+}
 E cudaEventCreate(cudaEvent_t* e) { return handle(e); }
 E cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return handle(e); }
 E cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
@@ -138,7 +149,11 @@ E cudaEventRecordWithFlags(cudaEvent_t e, cudaStream_t st, unsigned) { return wo
 E cudaEventSynchronize(cudaEvent_t e) { return note(EVENT_SYNC, nullptr, (uintptr_t)e); }
 E cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return handle(s); }
 E cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-E cudaStreamSynchronize(cudaStream_t st) { return note(STREAM_SYNC, st); }
+E cudaStreamSynchronize(cudaStream_t st) {
+  State& s = state();
+  s.kept = std::min(s.kept, s.threshold > s.live ? s.threshold - s.live : 0);
+  return note(STREAM_SYNC, st);
+}
 E cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) { return note(STREAM_WAIT, st, (uintptr_t)e); }
 E cudaDeviceSynchronize() { return cudaSuccess; }
 E cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {

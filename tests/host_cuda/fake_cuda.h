@@ -24,7 +24,12 @@ struct State {
   long fail_at = -1;     // the work call (counted from `work`) that fails; -1: none
   bool ones = false;     // copies of reduction results to the host read as 1.0
   size_t live = 0, high = 0;    // device bytes allocated now, and at most
+  size_t kept = 0;              // bytes given back that the pool still holds (never used again)
+  size_t threshold = 0;         // of the pool: what it may hold when a stream is waited for
+  size_t foreign = 0;           // bytes of other users of the device
   size_t total = 1ull << 38;    // bytes of the device
+  int trims = 0, refused = 0;   // calls that gave kept bytes back, allocations that failed
+  int host_blocks = 0;          // pinned blocks allocated now
 };
 State& state();
 

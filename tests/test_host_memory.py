@@ -35,6 +35,11 @@ def program(tmp_path_factory):
     return make
 
 
+def test_kept_memory_is_bounded_and_given_back(program):
+    r = subprocess.run([program("pool_limits")], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:]
+
+
 def test_solve_that_ends_early_leaves_nothing_running(program):
     r = subprocess.run([program("early_end")], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout[-2000:]
