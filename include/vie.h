@@ -244,9 +244,10 @@ vie_status vie_solve(vie_problem* P, const void* rhs, void* J, const vie_solve_o
  * J and field_out must not overlap (VIE_EINVAL).  Asynchronous on stream. */
 vie_status vie_eval_scattered(vie_problem* P, const void* J, void* field_out, int nrhs, void* stream);
 
-/* Device bytes a problem of this shape holds (medium, kernels, apply workspace
- * for nrhs right-hand sides, FP32 Krylov basis of length restart); used for
- * admission by memory budget.  has_mu: 1 for Maxwell with mu. */
+/* The most device bytes a problem of this shape holds at a time: set-up scratch,
+ * medium, kernels, a mixed solve (apply workspace for nrhs right-hand sides, FP32 Krylov
+ * basis of length restart for a lockstep group of them) and the scattered field after
+ * it; used for admission by memory budget.  has_mu: 1 for Maxwell with mu. */
 size_t vie_problem_bytes(int kind, int n, int nrhs, int restart, int has_mu);
 
 /* Release every allocation of the handle, stream-ordered on the stream the

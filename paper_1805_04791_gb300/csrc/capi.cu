@@ -359,21 +359,21 @@ vie_status vie_eval_scattered(vie_problem* P, const void* J, void* field_out, in
 
 size_t vie_problem_bytes(int kind, int n, int nrhs, int restart, int has_mu) {
   if (n < 1 || nrhs < 1 || restart < 1) return 0;
-  const size_t N = (size_t)n * n * n;
-  const size_t nk = (size_t)conv_half(n);
-  const size_t O3 = (nk + 1) * (nk + 1) * (nk + 1);
-  const int c = (kind == VIE_MAXWELL && has_mu) ? 6 : 3;
-  const int nsym = kind == VIE_MAXWELL ? 10 : 9;
-  size_t held = 144 * N * (has_mu ? 2 : 1);  // H: 6 entries, FP64 + FP32
-  held += 16 * O3 * nsym;                    // raw symbol octants
-  held += 24 * O3 * 18;                      // apply + eval kernel sets, FP64 + FP32
-  held += 96 * N * (has_mu ? 2 : 1) + 16 * O3 * (kind == VIE_MAXWELL ? 9 : 6);  // double-word copies (mixed solve)
-  // allowance for set-up scratch (the octant line operators hold less)
-  const size_t setup = held + 16 * (27 * N + 8 * nk * nk * nk);
-  // steady state: FP64 apply workspace, mixed-precision Krylov group
-  size_t steady = held + apply_workspace_bytes(n, (int)nk, c, nrhs, VIE_FP64);
-  steady += (size_t)nrhs * c * N * (8 * (size_t)(restart + 1) + 16 * 2 + 8);
-  return setup > steady ? setup : steady;
+  const bool mx = kind == VIE_MAXWELL, mu = mx && has_mu;
+  const size_t N = (size_t)n * n * n, nk = (size_t)conv_half(n), media = mu ? 2 : 1;
+  const size_t O = nk + 1, O3 = O * O * O, S = 3 * (size_t)n / 2 + 1;
+  const int c = mu ? 6 : 3, narr = mu ? 9 : 6, nfield = mx ? 9 : 3;
+  const size_t medium = 144 * N * media + 64 * 1024;  // H: 6 entries, FP64 + FP32; flags, line table
+  const size_t bases = 16 * O3 * 4;
+  // set-up scratch (compute_symbols): two line-operator buffers, the table of G^, line tables
+  const size_t scratch = 32 * (S * S * O + S * O * O) + 48 * S * S + 1080 * 2 * (size_t)n;
+  // a mixed solve of nrhs right-hand sides: kernels, double-word copies, Krylov workspace
+  const size_t solve = medium + bases + 40 * O3 * narr + 96 * N * media + krylov_bytes((long long)(c * N), restart, nrhs);
+  // the scattered field after it: set-up of the base that the operator does not need,
+  // beside the solve's workspace; then its kernels and its own (E and H: six components)
+  const size_t base = solve + apply_workspace_bytes(n, (int)nk, c, nrhs, VIE_FP64) + (mu ? 0 : scratch);
+  const size_t field = solve + 24 * O3 * nfield + apply_workspace_bytes(n, (int)nk, mx ? 6 : 3, nrhs, VIE_FP64);
+  return std::max(medium + bases + scratch, std::max(base, field));
 }
 
 vie_status vie_tune(vie_problem* P, int precision, int* variant, void* stream) {

@@ -1096,9 +1096,15 @@ static size_t group_bytes_per_rhs(long long L, int m, bool mixed) {
          2 * (m + 4)) + arn + 16 * 256;
 }
 
+static size_t group_bytes(long long L, int m, bool mixed, int nb) {
+  return group_bytes_per_rhs(L, m, mixed) * nb + 32 * 4096;
+}
+
+size_t krylov_bytes(long long L, int m, int nrhs) { return group_bytes(L, m, true, std::min(nrhs, kGroupMax)); }
+
 static vie_status ensure_group(vie_problem* P, int m, bool mixed, int nb, Group& g, cudaStream_t st) {
   const long long L = (long long)P->ncomp * P->n * P->n * P->n;
-  const size_t need = group_bytes_per_rhs(L, m, mixed) * nb + 32 * 4096;
+  const size_t need = group_bytes(L, m, mixed, nb);
   if (P->ks.bytes < need) {
     dfree(P->ks.buf, st);
     P->ks.buf = nullptr;

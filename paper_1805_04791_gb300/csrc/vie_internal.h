@@ -169,6 +169,8 @@ bool p3_schedule_ready(vie_problem* P, const KernelSet& K, int prec);
 // krylov.cu
 vie_status run_solve(vie_problem* P, const void* rhs, void* J, const vie_solve_opts* opt, vie_solve_info* info,
                      cudaStream_t st);
+// Bytes of the Krylov workspace of a mixed solve of nrhs right-hand sides of L values.
+size_t krylov_bytes(long long L, int m, int nrhs);
 vie_status run_rhs(vie_problem* P, const double* d, const double* p, int nrhs, void* out, cudaStream_t st);
 
 // Allow a kernel the device's full opt-in dynamic shared memory.  The attribute

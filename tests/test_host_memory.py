@@ -35,6 +35,13 @@ def program(tmp_path_factory):
     return make
 
 
+def test_problem_bytes_is_what_a_problem_holds(program):
+    """At least the most that create, a mixed solve and the scattered field hold together,
+    and at most 5 % and 256 KiB (small buffers) more."""
+    r = subprocess.run([program("problem_bytes")], capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, "\n".join(v for v in r.stdout.splitlines() if v.startswith("BAD"))
+
+
 def test_kept_memory_is_bounded_and_given_back(program):
     r = subprocess.run([program("pool_limits")], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout[-2000:]
