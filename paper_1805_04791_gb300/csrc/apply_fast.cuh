@@ -1725,16 +1725,16 @@ struct FastPath {
   // Helmholtz 642 and 687 us, E and H of reduced Maxwell 963 and 1128 us.
   template <int MODE>
   static vie_status p3_tile(V* B, int n, int C, const V* K, int nrhs, const V* tw, bool* done, cudaStream_t st) {
-    if constexpr (std::is_same<T, double>::value) {
+    if constexpr (std::is_same<T, double>::value && has_two_plan(M)) {
       TwoPlan tp;
-      if (make_two_plan(M, &tp)) {
-        const TwoArgs a = {n, MODE, C, 0, 0, nrhs, 0, nullptr, nullptr, nullptr, K, tw, nullptr, nullptr, B};
-        vie_status e = tp.R1 <= 16 ? two_pass_f64_16(3, tp, a, st) : two_pass_f64_24(3, tp, a, st);
-        *done = e == VIE_OK;
-        return e;
-      }
+      make_two_plan(M, &tp);
+      const TwoArgs a = {n, MODE, C, 0, 0, nrhs, 0, nullptr, nullptr, nullptr, K, tw, nullptr, nullptr, B};
+      vie_status e = tp.R1 <= 16 ? two_pass_f64_16(3, tp, a, st) : two_pass_f64_24(3, tp, a, st);
+      *done = e == VIE_OK;
+      return e;
+    } else {
+      return p3b_ok<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
     }
-    return p3b_ok<MODE, 8>(B, n, C, K, nrhs, tw, done, st);
   }
   template <int MODE>
   static vie_status p3_mode(int variant, V* B, int n, int C, const V* K, int nrhs, const V* tw, bool* done,

@@ -37,10 +37,10 @@ struct TwoPlan {
 };
 
 // Radices with a codelet in the run-time switches.
-inline bool two_radix(int r) { return r >= 4 && r <= 24 && r != 13 && r != 17 && r != 19 && r != 23; }
+constexpr bool two_radix(int r) { return r >= 4 && r <= 24 && r != 13 && r != 17 && r != 19 && r != 23; }
 
 // The most balanced split with R1 >= R2.
-inline bool make_two_plan(int M, TwoPlan* p) {
+constexpr bool make_two_plan(int M, TwoPlan* p) {
   for (int r2 = 24; r2 >= 4; --r2) {
     if (r2 * r2 > M || M % r2 || !two_radix(r2) || !two_radix(M / r2) || (M / r2 > 16 && r2 < 9)) continue;
     p->M = M;
@@ -50,6 +50,11 @@ inline bool make_two_plan(int M, TwoPlan* p) {
     return true;
   }
   return false;
+}
+
+constexpr bool has_two_plan(int M) {
+  TwoPlan p{};
+  return make_two_plan(M, &p);
 }
 
 // Whether the z pass has a two-step kernel for M: all but the double-word one
