@@ -299,8 +299,8 @@ vie_status vie_tune(vie_problem* P, int precision, int* variant, void* stream);
  * event before and after each of their kernel launches (on the launch stream;
  * no synchronisation), for at most cap applies.  vie_profile_end synchronises
  * the device, writes into ms[k] (k < nslots, host) the total milliseconds spent
- * in kernel slot k (0..4: the five passes of the pipeline, see apply.cu),
- * writes the number of recorded applies to *count, and stops recording. */
+ * in kernel slot k (0..4: the five passes of the pipeline, see apply.cu; where one
+ * kernel does the first two, FP32 at 2n = 64 and 96, its time is in slot 0), writes the number of recorded applies to *count, and stops recording. */
 vie_status vie_profile_begin(vie_problem* P, int cap);
 vie_status vie_profile_end(vie_problem* P, double* ms, int nslots, int* count);
 

@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kRedThreads) k_arn_axpy(TB* __restrict__ V, lo
     for (int q = 0; q < W; ++q)
 #pragma unroll
       for (int u = 0; u < 4; ++u) sx[q][u] = sy[q][u] = 0;
-    // N basis loads in flight, then their products into N / 2 (or 1) partial sums
+    // N basis loads in flight, then their products into four partial sums
     auto terms = [&](int i, auto nc) {
       constexpr int N = decltype(nc)::value;
       if (packed) {
@@ -1207,7 +1207,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dots4(Dots4 d, long long L, dou
   block_sums<K>(ar, ai, partial + blockIdx.x, gridDim.x);
 }
 
-// y = a0 x0 + a1 x1 (+ a2 x2 if N = 3; y may alias x0), four elements' loads in flight.
+// y = a0 x0 + a1 x1 (+ a2 x2 if N = 3; y may be any of them), four elements' loads in flight.
 template <int N>
 __global__ void __launch_bounds__(256) k_lincomb(double2* y, const double2* x0, double2 a0, const double2* x1, double2 a1,
                                                  const double2* x2, double2 a2, long long L) {
