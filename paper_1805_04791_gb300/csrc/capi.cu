@@ -137,6 +137,7 @@ void pinned_give(void* p) {
 }
 
 vie_status cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();  // the runtime keeps it for the next check otherwise, which would report it again
   g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
   return e == cudaErrorMemoryAllocation ? VIE_ENOMEM : VIE_ECUDA;
 }

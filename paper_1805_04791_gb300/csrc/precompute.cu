@@ -479,14 +479,25 @@ __global__ void __launch_bounds__(256) k_combine(const double2* __restrict__ bas
 static vie_status combine(vie_problem* P, KernelSet& K, int mode, const CombineDesc& cd, double diag_add,
                           int diag_mask, cudaStream_t st) {
   const long long O = P->nk + 1, O3 = O * O * O;
+  double2* oct64 = nullptr;
+  float2* oct32 = nullptr;
+  cudaError_t e = dalloc((void**)&oct64, sizeof(double2) * cd.narr * O3, st);
+  if (e == cudaSuccess) e = dalloc((void**)&oct32, sizeof(float2) * cd.narr * O3, st);
+  if (e == cudaSuccess) {
+    const unsigned tiles = (unsigned)((O + 31) / 32);
+    k_combine<<<dim3(tiles, tiles, (unsigned)O), dim3(32, 8), 0, st>>>(P->base_oct, oct64, oct32, (int)O, cd, diag_add,
+                                                                       diag_mask);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) {  // the set stays as it was: its arrays say whether it is built
+    dfree(oct64, st);
+    dfree(oct32, st);
+    return cuda_fail(e, "kernel set");
+  }
   K.mode = mode;
   K.narr = cd.narr;
-  VIE_CK(dalloc((void**)&K.oct64, sizeof(double2) * cd.narr * O3, st));
-  VIE_CK(dalloc((void**)&K.oct32, sizeof(float2) * cd.narr * O3, st));
-  const unsigned tiles = (unsigned)((O + 31) / 32);
-  k_combine<<<dim3(tiles, tiles, (unsigned)O), dim3(32, 8), 0, st>>>(P->base_oct, K.oct64, K.oct32, (int)O, cd,
-                                                                     diag_add, diag_mask);
-  VIE_CK(cudaGetLastError());
+  K.oct64 = oct64;
+  K.oct32 = oct32;
   return VIE_OK;
 }
 

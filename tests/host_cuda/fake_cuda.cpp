@@ -33,7 +33,9 @@ static cudaError_t note(Op op, cudaStream_t st, uintptr_t ev = 0) {
 }
 static cudaError_t take(void** p, size_t bytes) {
   State& s = state();
-  if (s.live + s.kept + s.foreign + bytes > s.total) {
+  const long nr = s.allocations++;
+  const bool refuse = s.refuse_at >= 0 && (nr == s.refuse_at || nr == s.refuse_at + 1);
+  if (refuse || s.live + s.kept + s.foreign + bytes > s.total) {
     ++s.refused;
     g_last = cudaErrorMemoryAllocation;
     return g_last;

@@ -28,6 +28,8 @@ struct State {
   size_t threshold = 0;         // of the pool: what it may hold when a stream is waited for
   size_t foreign = 0;           // bytes of other users of the device
   size_t total = 1ull << 38;    // bytes of the device
+  long allocations = 0;         // calls so far, the ones that failed included
+  long refuse_at = -1;          // the allocation that fails, tried twice in a row; -1: none
   int trims = 0, refused = 0;   // calls that gave kept bytes back, allocations that failed
   int host_blocks = 0;          // pinned blocks allocated now
 };

@@ -47,6 +47,11 @@ def test_kept_memory_is_bounded_and_given_back(program):
     assert r.returncode == 0, r.stdout[-2000:]
 
 
+def test_calls_work_after_a_refused_allocation(program):
+    r = subprocess.run([program("refused_memory")], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:]
+
+
 def test_solve_that_ends_early_leaves_nothing_running(program):
     r = subprocess.run([program("early_end")], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout[-2000:]
