@@ -457,8 +457,8 @@ static vie_status run_apply_t(vie_problem* P, const KernelSet& K, const void* in
   FastSel fs = fast_select(fast_grid(P), K.mode, with_identity);
   if (Prec<T>::id == VIE_DF64) {
     // double-word fast kernels exist for 2n = 256 and the operator's kernel sets
-    // only (z pass 1.19 ms, two-step 1.34); its register-resident P5 (254
-    // registers, one CTA per SM) is slower than the two-step one (0.32 ms)
+    // only (z pass 1.33 ms, two-step 1.49); its register-resident P5 (254
+    // registers, one CTA per SM) is slower than the two-step one (0.33 ms)
     if (!(M == 256 && fs.p1 && (K.mode == KM_SYM3 || K.mode == KM_MAXWELL6))) fs = FastSel();
     fs.p5 = false;
   }

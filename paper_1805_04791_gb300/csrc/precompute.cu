@@ -225,9 +225,9 @@ __global__ void k_ghat_table(double2* tab, int jmax, double dk, double w, double
 // exchanging axes (G^ is radial): 1, -k_z^2, -k_x k_y and i k_z, z being the
 // axis that is not like the other two.
 // Measured, 192^3 reduced Maxwell problem: 302 ms for seven symbols on whole cubes
-// (279 ms of cube transforms, 21 ms to fill them); three bases here take 10.3 ms
-// (29.5 with the double-word sums and products of twice the instructions, 12.3
-// without the pairing in k_axis; Helmholtz 64^3 0.43 -> 0.32 ms by it).
+// (279 ms of cube transforms, 21 ms to fill them); three bases here take 10.8 ms
+// (29.5 with a normalisation after every double-word operation; the pairing in k_axis
+// saved a sixth here and a quarter at Helmholtz 64^3, now 0.37 ms).
 enum Base { BASE_1 = 0, BASE_ZZ, BASE_XY, BASE_DZ, BASE_COUNT };
 
 static int base_of(int sym) {

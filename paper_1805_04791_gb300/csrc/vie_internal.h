@@ -218,7 +218,7 @@ inline cudaError_t allow_smem(K* kernel, bool max_carveout = false) {
 static const unsigned long long kLaunchAfterThreads = 152 * 448;
 // FP64 passes and reductions are launched plainly too: bound by the FP64 pipe, they
 // are long for their grids and lose by it (FP64 apply at 32^3 142 us, 197 launched so;
-// double-word 70 us, 59 launched so).
+// double-word 63.5 us, 61.3 launched so).
 template <typename T> constexpr bool kOverlap = !std::is_same<T, double>::value && !std::is_same<T, double2>::value;
 template <bool OVERLAP, typename... P, typename... A>
 inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {

@@ -18,10 +18,12 @@
 //
 // Measured against the Stockham passes (whole apply): FP32 reduced Maxwell 70^3
 // 271 -> 136 us, 150^3 2.57 -> 1.01 ms, 220^3 8.46 -> 3.15 ms; FP64 Helmholtz 70^3
-// 2.54 -> 1.91 ms; double-word 64^3 0.54 -> 0.44, 96^3 1.44 -> 1.10 ms (with the
-// same arithmetic).  FP32 at 150^3: the x and y passes move their bytes at 3.8 to
-// 4.5 TB/s; the z pass (0.57 ms) waits for shared memory and its barriers at 24
-// warps an SM.  FP64 and double-word passes are bound by their pipes.
+// 2.54 -> 1.91 ms; double-word 64^3 0.54 -> 0.44, 96^3 1.44 -> 1.10 ms (the same
+// arithmetic on both sides; 0.46 and 1.17 ms with today's).  FP32 at 150^3: the x and y
+// passes move their bytes at 3.8 to 4.5 TB/s; the z pass (0.57 ms) issues 55 % of the
+// cycles at 24 warps an SM, waiting in equal parts for its barriers, its loads and FP32
+// latencies.  FP64 passes keep the FP64 pipe 81 - 84 % busy (70^3), the double-word z
+// pass the FP32 pipe 63 % (96^3).
 #pragma once
 
 #include <type_traits>
